@@ -316,6 +316,16 @@ def _fill_positions(pos, g):
     pos.copy_(gaps.cumsum(-1, dtype=torch.int32))
 
 
+def _decode_step(s, t, l, count):
+    """Step t of layers [l, l + count)."""
+    q, kn, vn, out = (x[t, l:l + count] for x in (s.q, s.kn, s.vn, s.out))
+    if s.paged:
+        voxzip_decode_step_paged(s.desc, s.paged, l, count, q, kn, vn, s.new_pos[t], s.gamma, out, max_len=s.n + t + 1)
+    else:
+        voxzip_decode_step(s.desc, l, count, q, kn, vn, s.new_pos[t], s.k, s.v, s.score, s.pos, s.len, s.gamma, out,
+                           max_len=s.n + t + 1)
+
+
 def _prepare_decode(c, seed):
     s, g, dt = State(), _generator(seed), DTYPES[c["dtype"]]
     B, L, H, D, steps = c["batch"], c["layers"], c["kv_heads"], c["head_dim"], c["steps"]
@@ -347,27 +357,17 @@ def _prepare_decode(c, seed):
     s.out = torch.empty_like(s.q)
     s.gamma, s.steps, s.n, s.graph = c["gamma"], steps, max(lens), None
 
-    def step(t, l, count):
-        q, kn, vn, out = (x[t, l:l + count] for x in (s.q, s.kn, s.vn, s.out))
-        if s.paged:
-            voxzip_decode_step_paged(desc, s.paged, l, count, q, kn, vn, s.new_pos[t], s.gamma, out,
-                                     max_len=s.n + t + 1)
-        else:
-            voxzip_decode_step(desc, l, count, q, kn, vn, s.new_pos[t], s.k, s.v, s.score, s.pos, s.len, s.gamma, out,
-                               max_len=s.n + t + 1)
-
-    s.step = step
     if c["launch"] != "eager":
         s.score.zero_()
         s.len.copy_(s.len0)
-        step(0, 0, 1 if c["launch"] == "layers" else L)  # loads the kernels before the capture
+        _decode_step(s, 0, 0, 1 if c["launch"] == "layers" else L)  # loads the kernels before the capture
         torch.cuda.synchronize()
         s.graph = torch.cuda.CUDAGraph()
         with torch.cuda.graph(s.graph):
             s.len.copy_(s.len0)
             for t in range(steps):
                 for l in range(L if c["launch"] == "layers" else 1):
-                    step(t, l, 1 if c["launch"] == "layers" else L)
+                    _decode_step(s, t, l, 1 if c["launch"] == "layers" else L)
     # decayed sums of the softmax mass a step adds
     s.score.exponential_(1.0, generator=g).mul_(c["q_heads"] / H / (max(1, s.n) * (1.005 - c["gamma"])))
     s.len.copy_(s.len0)
@@ -472,7 +472,7 @@ def run(s):
             s.graph.replay()
         else:
             s.len.copy_(s.len0)
-            s.step(0, 0, s.desc.layers)
+            _decode_step(s, 0, 0, s.desc.layers)
         return dict(out=s.out, score=s.score, k=s.k, v=s.v, pos=s.pos, len=s.len)
     if s.kind == "evict":
         s.live.copy_(s.before)

@@ -8,9 +8,16 @@
 //   phase K  S = K_tile Q^T on the tensor cores (mma.sync m16n8k16, tokens as M, the group's
 //            query heads as N); scaled logits kept in shared memory; a running per-head maximum
 //            and normaliser (online softmax statistics; kept only when S = 1).
-//   phase V  p = 2^(logit - max_cta); O^T += V_tile^T P^T on the tensor cores. A CTA that holds the
+//   phase V  p = 2^(logit - max); O^T += V_tile^T P^T on the tensor cores. A CTA that holds the
 //            whole unit (S = 1) already has the final statistics: it rewrites the scores tile by
-//            tile as gamma * s + sum_h p_h / Z_h. In a cluster p is kept in shared memory instead.
+//            tile as gamma * s + sum_h p_h / Z_h. In a cluster p is kept in shared memory instead, and
+//            is taken with the warp's own maximum, so that no barrier stands between the phases.
+// A short launch (one layer of a token, a few tiles per CTA) is bound by the latency of this chain,
+// not by HBM: length, first tile, two phases, partial sums, cluster barrier, exchange. With the ring
+// set up before the dependency wait, a warp's own maximum, P^T taken from the logits in the B operand's
+// layout (no round trip through shared memory) and partial sums by 16-byte loads, a layer's launch at
+// 10-min 20x (32 CTAs) went from 5.2 to 4.7 us with its rows in L2, and the request of a 30-s clip
+// (31 steps, all layers) from 369 to 348 us.
 // As each tile issues, the tile one ring-depth ahead is requested into L2 (bulk prefetch), so an
 // SM keeps more bytes in flight than its rings hold. Launches are programmatic dependents of the
 // previous kernel on the stream: a CTA sets up (barriers, the L2 prefetch of its first tiles)
@@ -94,10 +101,8 @@ struct Layout {
     static constexpr int kOwBytes = kConsumerWarps * kGP * kOStride * 4;
     static constexpr int kRingAlloc = kRingBytes > kOwBytes ? kRingBytes : (kOwBytes + 1023) / 1024 * 1024;
     static constexpr int kBarOff = kRingAlloc;                 // full[kStages], empty[kStages]
-    static constexpr int kPbufOff = kBarOff + 2 * kStages * 8;
-    static constexpr int kPbufBytes = kConsumerWarps * 16 * kGP * 2;
-    static constexpr int kStatOff = kPbufOff + kPbufBytes;     // m_w, z_w [warps][kGP]; m_cta, z_cta [kGP]; fac [S][kGP]
-    static constexpr int kStatFloats = (2 * kConsumerWarps + 2 + kMaxCluster) * kGP;
+    static constexpr int kStatOff = kBarOff + 2 * kStages * 8;  // m_w, z_w, f_w [warps][kGP]; m_cta, z_cta [kGP]; fac [S][kGP]
+    static constexpr int kStatFloats = (3 * kConsumerWarps + 2 + kMaxCluster) * kGP;
     static constexpr int kLgOff = kStatOff + kStatFloats * 4;  // logits / p [chunk_cap][kGP] fp32, then old scores
     static size_t bytes(int chunk_cap) {  // + the pool row of each tile (paged)
         return 1024 + (size_t)kLgOff + (size_t)chunk_cap * kGP * 4 + (size_t)chunk_cap * 4 +
@@ -108,6 +113,10 @@ struct Layout {
 __device__ __forceinline__ uint32_t swz(int row, int chunk) {  // byte offset in a 128B-swizzled box
     return (uint32_t)(row * 128 + ((chunk ^ (row & 7)) << 4));
 }
+
+// Row of local token i in the logits: within 16 tokens, 8b + 2q + a goes to row 8b + 4a + q, so that
+// phase V's reads (a lane group per q, a and b fixed) take four consecutive rows and no bank twice.
+__device__ __forceinline__ int lg_row(int i) { return (i & ~7) | ((i & 1) << 2) | ((i >> 1) & 3); }
 
 // kCluster: launched in clusters of S > 1 CTAs (else one CTA holds the whole unit).
 // kPaged: K/V rows live in page pools (see paged.cuh).
@@ -132,12 +141,12 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
     uint8_t *stages = smem + Lay::kStagesOff;
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + Lay::kBarOff);
     uint64_t *empty = full + kStages;
-    uint8_t *pbuf = smem + Lay::kPbufOff + warp * 16 * GP * 2;
     float *o_w = reinterpret_cast<float *>(stages);            // [warps][GP][D], valid after the ring drains
     float *o_cta = o_w;                                        // the sum over warps lands in warp 0's slot
     float *m_w = reinterpret_cast<float *>(smem + Lay::kStatOff);
     float *z_w = m_w + kConsumerWarps * GP;
-    float *m_cta = z_w + kConsumerWarps * GP;                  // this CTA's per-head maximum (log2 units)
+    float *f_w = z_w + kConsumerWarps * GP;                    // 2^(m_w - m_cta); at the end the scores' factors
+    float *m_cta = f_w + kConsumerWarps * GP;                  // this CTA's per-head maximum (log2 units)
     float *z_cta = m_cta + GP;                                 // and normaliser relative to it
     float *fac = z_cta + GP;                                   // [S][GP]: 2^(m_r - m) / Z; 0 for padding heads
     float *lg = reinterpret_cast<float *>(smem + Lay::kLgOff);
@@ -147,6 +156,15 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
     const UnitIdx ui = unit_of(blockIdx.y, p.B, p.L, p.Hkv, p.layer_begin);
     const int64_t act_row = (int64_t)ui.l_local * p.B + ui.b;
     const int64_t row_base = ui.cache_unit * p.C;
+    // The ring is set up before the dependency wait, so that the producer's first load waits only for
+    // the unit's length, and not for what the consumer warps load first.
+    if (tid == 0) {
+        for (int s = 0; s < kStages; ++s) {
+            ptx::mbar_init(&full[s], 1);
+            ptx::mbar_init(&empty[s], kConsumerWarps);
+        }
+        ptx::fence_mbar_init();
+    }
     // While this unit's length is read, pull the first tiles of the range the launch's length hint
     // predicts into L2 (exact when the unit is as long as the hint; otherwise a few wasted KB).
     if (!kPaged && warp == kConsumerWarps && lane == 0) {
@@ -154,6 +172,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
         const int rows = min(kStages * kTile, p.C - est_j0);
         if (rows > 0) ptx::prefetch_l2(p.k_cache + (row_base + est_j0) * D, (uint32_t)rows * D * 2);
     }
+    __syncthreads();
     // Launched as a programmatic dependent of the previous kernel on the stream, the CTA may start
     // before that kernel ends: everything from here on reads what it wrote (lengths, pages,
     // cache rows, scores, queries), so wait for its completion. (The prefetch above is a hint.)
@@ -247,13 +266,6 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
         if (lane == 0) p.pos[row_base + n - 1] = pos_new;
         appended = true;
     };
-    if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) {
-            ptx::mbar_init(&full[s], 1);
-            ptx::mbar_init(&empty[s], kConsumerWarps);
-        }
-        ptx::fence_mbar_init();
-    }
     // The old scores of this CTA's tokens travel to shared memory while the tiles stream.
     if (warp < kConsumerWarps) {
         const float *src = p.score + row_base + j0;
@@ -262,7 +274,6 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
                          : "memory");
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    __syncthreads();
 
     bool ok = true;
     if (warp == kConsumerWarps) {
@@ -317,6 +328,15 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) mx[nt][0] = mx[nt][1] = -INFINITY, zx[nt][0] = zx[nt][1] = 0.f;
         const int r0 = warp * 16;
+        // The largest of one head's per-warp maxima m[w * GP], and f[w] = 2^(m_w - it).
+        auto warp_factors = [](const float *m, float (&f)[kConsumerWarps]) {
+            float mm = -INFINITY;
+#pragma unroll
+            for (int w = 0; w < kConsumerWarps; ++w) mm = fmaxf(mm, f[w] = m[w * GP]);
+#pragma unroll
+            for (int w = 0; w < kConsumerWarps; ++w) f[w] = f[w] == -INFINITY ? 0.f : exp2f(f[w] - mm);
+            return mm;
+        };
 
         // Phase K: logits of this warp's 16 tokens of every tile.
         for (int t = 0; t < ntiles && ok; ++t) {
@@ -377,9 +397,9 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
                                         exp2f(lb[j] - m_new);
                         mx[nt][j] = m_new;
                     }
-                    if (va) *reinterpret_cast<float2 *>(lg + (lt0 + g) * GP + nt * 8 + 2 * qd) = make_float2(la[0], la[1]);
-                    if (vb)
-                        *reinterpret_cast<float2 *>(lg + (lt0 + g + 8) * GP + nt * 8 + 2 * qd) = make_float2(lb[0], lb[1]);
+                    float *l = lg + lg_row(lt0 + g) * GP + nt * 8 + 2 * qd;
+                    if (va) *reinterpret_cast<float2 *>(l) = make_float2(la[0], la[1]);
+                    if (vb) *reinterpret_cast<float2 *>(l + 8 * GP) = make_float2(lb[0], lb[1]);
                 }
                 if (patch) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // before the slot's next TMA
             }
@@ -387,7 +407,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
             if (lane == 0) ptx::mbar_arrive(&empty[s]);
         }
         if (patcher && !appended) append();  // phase K ended early (a wait gave up)
-        // Per-head statistics of the warp (merge over the 8 lanes that share qd), then of the CTA.
+        // Per-head statistics of the warp: merge over the 8 lanes that share qd.
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -396,50 +416,67 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
 #pragma unroll
                 for (int off = 4; off <= 16; off <<= 1) {
                     const float mo = __shfl_xor_sync(0xffffffffu, m, off);
-                    const float zo = __shfl_xor_sync(0xffffffffu, z, off);
                     const float mm = fmaxf(m, mo);
-                    z = (m == -INFINITY ? 0.f : z * exp2f(m - mm)) + (mo == -INFINITY ? 0.f : zo * exp2f(mo - mm));
+                    if (!clustered) {
+                        const float zo = __shfl_xor_sync(0xffffffffu, z, off);
+                        z = (m == -INFINITY ? 0.f : z * exp2f(m - mm)) + (mo == -INFINITY ? 0.f : zo * exp2f(mo - mm));
+                    }
                     m = mm;
                 }
+                mx[nt][j] = m;
                 if (g == 0) {
                     m_w[warp * GP + nt * 8 + 2 * qd + j] = m;
-                    z_w[warp * GP + nt * 8 + 2 * qd + j] = z;
+                    if (!clustered) z_w[warp * GP + nt * 8 + 2 * qd + j] = z;
                 }
             }
-        asm volatile("cp.async.wait_all;" ::: "memory");  // this thread's old scores have landed
-        asm volatile("bar.sync 1, %0;" ::"r"(kConsumerWarps * 32) : "memory");
-        if (tid < GP) {
-            float m = -INFINITY, z = 0.f;
+        // From here on a lane serves head nt * 8 + g: mc is the maximum its probabilities are taken
+        // with, rc the normaliser's reciprocal (S = 1).
+        float mc[NT], rc[NT], zv[NT];
+        if constexpr (!kCluster) {
+            // A CTA that holds the whole unit has its final statistics now.
+            asm volatile("cp.async.wait_all;" ::: "memory");  // this thread's old scores have landed
+            asm volatile("bar.sync 1, %0;" ::"r"(kConsumerWarps * 32) : "memory");
+            if (tid < GP) {
+                float m = -INFINITY, z = 0.f;
 #pragma unroll
-            for (int w = 0; w < kConsumerWarps; ++w) m = fmaxf(m, m_w[w * GP + tid]);
+                for (int w = 0; w < kConsumerWarps; ++w) m = fmaxf(m, m_w[w * GP + tid]);
 #pragma unroll
-            for (int w = 0; w < kConsumerWarps; ++w) {
-                const float mw = m_w[w * GP + tid];
-                if (mw != -INFINITY) z += z_w[w * GP + tid] * exp2f(mw - m);
+                for (int w = 0; w < kConsumerWarps; ++w) {
+                    const float mw = m_w[w * GP + tid];
+                    if (mw != -INFINITY) z += z_w[w * GP + tid] * exp2f(mw - m);
+                }
+                m_cta[tid] = m;
+                fac[tid] = tid < p.G ? 1.f / z : 0.f;
             }
-            m_cta[tid] = m;
-            z_cta[tid] = z;
+            asm volatile("bar.sync 1, %0;" ::"r"(kConsumerWarps * 32) : "memory");
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                mc[nt] = m_cta[nt * 8 + g];
+                rc[nt] = fac[nt * 8 + g];
+                zv[nt] = 0.f;
+            }
+        } else {
+            // In a cluster every warp goes on with its own maximum: no barrier stands between its last
+            // K tile and its first V tile, and the warps' partial results are rescaled when they are
+            // summed. (A maximum of -inf, from a warp with no token or logits all -inf, counts as 0.)
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) {
+                const float m0 = __shfl_sync(0xffffffffu, mx[nt][0], g >> 1);
+                const float m1 = __shfl_sync(0xffffffffu, mx[nt][1], g >> 1);
+                const float m = (g & 1) ? m1 : m0;
+                mc[nt] = m == -INFINITY ? 0.f : m;
+                rc[nt] = 0.f;
+                zv[nt] = 0.f;
+            }
         }
-        // A CTA that holds the whole unit has its final statistics now.
-        if (!clustered && tid < GP) fac[tid] = tid < p.G ? 1.f / z_cta[tid] : 0.f;
-        asm volatile("bar.sync 1, %0;" ::"r"(kConsumerWarps * 32) : "memory");
 
-        // Phase V: probabilities with the CTA maximum, P V on the tensor cores; without a cluster
-        // also the score update (Eq. 6), else p is kept for it.
+        // Phase V: probabilities, P V on the tensor cores; without a cluster also the score update
+        // (Eq. 6), else p is kept for it.
         float oacc[kKSteps][NT][4];
 #pragma unroll
         for (int i = 0; i < kKSteps; ++i)
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) oacc[i][nt][0] = oacc[i][nt][1] = oacc[i][nt][2] = oacc[i][nt][3] = 0.f;
-        float mc[NT][2], rc[NT][2], zv[NT][2];
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                mc[nt][j] = m_cta[nt * 8 + 2 * qd + j];
-                rc[nt][j] = clustered ? 0.f : fac[nt * 8 + 2 * qd + j];
-                zv[nt][j] = 0.f;
-            }
         float *sc = p.score + row_base + j0;
         for (int t = 0; t < ntiles && ok; ++t) {
             const int i = ntiles + t, s = i % kStages;
@@ -450,35 +487,45 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
             const int lt0 = t * kTile + r0;
             if (lt0 < cnt) {
                 uint8_t *stage = stages + s * Lay::kStageBytes;
+                // P^T as the B operand, straight from the logits: lane (g, qd) holds head nt * 8 + g of
+                // tokens 2 qd, 2 qd + 1, 2 qd + 8 and 2 qd + 9.
+                uint32_t pb[NT][2];
+                float add[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    const int lt = lt0 + g + half * 8;
-                    const bool valid = lt < cnt;
-                    float add = 0.f;
+                for (int nt = 0; nt < NT; ++nt) {
+                    float pr[4];
 #pragma unroll
-                    for (int nt = 0; nt < NT; ++nt) {
-                        float p0 = 0.f, p1 = 0.f;
-                        if (valid) {
-                            const float2 l = *reinterpret_cast<const float2 *>(lg + lt * GP + nt * 8 + 2 * qd);
-                            p0 = exp2f(l.x - mc[nt][0]);
-                            p1 = exp2f(l.y - mc[nt][1]);
-                            if (clustered) {
-                                *reinterpret_cast<float2 *>(lg + lt * GP + nt * 8 + 2 * qd) = make_float2(p0, p1);
-                                zv[nt][0] += p0;
-                                zv[nt][1] += p1;
-                            } else {
-                                add += p0 * rc[nt][0] + p1 * rc[nt][1];
-                            }
+                    for (int e = 0; e < 4; ++e) {
+                        const int lt = lt0 + 2 * qd + (e & 1) + (e >> 1) * 8;
+                        pr[e] = 0.f;
+                        if (lt < cnt) {
+                            float *l = lg + (lt0 + qd + 4 * e) * GP + nt * 8 + g;  // lg_row(lt)
+                            pr[e] = exp2f(*l - mc[nt]);
+                            if (clustered) *l = pr[e];
                         }
-                        *reinterpret_cast<uint32_t *>(pbuf + (g + half * 8) * GP * 2 + (nt * 8 + 2 * qd) * 2) =
-                            ptx::pack_bf16(p0, p1);
                     }
-                    if (!clustered) {  // Eq. 6: A = gamma * [A, 0] + sum over the heads (a token's four lanes)
-                        add += __shfl_xor_sync(0xffffffffu, add, 1);
-                        add += __shfl_xor_sync(0xffffffffu, add, 2);
-                        if (valid && qd == 0 && VOXZIP_IN_RANGE(p.status, j0 + lt < p.C))
-                            sc[lt] = lt == jn ? add : p.gamma * s_old[lt] + add;
+                    if (clustered) {
+                        zv[nt] += (pr[0] + pr[1]) + (pr[2] + pr[3]);
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) add[e] += pr[e] * rc[nt];
                     }
+                    pb[nt][0] = ptx::pack_bf16(pr[0], pr[1]);
+                    pb[nt][1] = ptx::pack_bf16(pr[2], pr[3]);
+                }
+                if (!clustered) {
+                    // Eq. 6: A = gamma * [A, 0] + sum over the heads. The 8 lanes that share qd sum their
+                    // four tokens' shares by halves: lane bits 4 and 3 choose the token a lane ends up with.
+                    const bool hi = lane & 16, odd = lane & 8;
+                    float a0 = hi ? add[2] : add[0], a1 = hi ? add[3] : add[1];
+                    a0 += __shfl_xor_sync(0xffffffffu, hi ? add[0] : add[2], 16);
+                    a1 += __shfl_xor_sync(0xffffffffu, hi ? add[1] : add[3], 16);
+                    float a = odd ? a1 : a0;
+                    a += __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 8);
+                    a += __shfl_xor_sync(0xffffffffu, a, 4);
+                    const int lt = lt0 + 2 * qd + (odd ? 1 : 0) + (hi ? 8 : 0);
+                    if (!(lane & 4) && lt < cnt && VOXZIP_IN_RANGE(p.status, j0 + lt < p.C))
+                        sc[lt] = lt == jn ? a : p.gamma * s_old[lt] + a;
                 }
                 // Rows past the range may hold anything; zero them so 0 * garbage cannot be NaN.
                 bool wrote = false;
@@ -497,10 +544,6 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
                 }
                 if (wrote) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
-                uint32_t pb[NT][2];
-#pragma unroll
-                for (int nt = 0; nt < NT; ++nt)
-                    ptx::ldsm_x2_t(ptx::smem_u32(pbuf + (lane & 15) * GP * 2 + nt * 16), pb[nt][0], pb[nt][1]);
                 const uint32_t base = ptx::smem_u32(stage);
                 const int mi = lane >> 3;
                 const int vrow = r0 + (lane & 7) + (mi >> 1) * 8;
@@ -519,20 +562,30 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&empty[s]);
         }
-        if (clustered) {  // per-head sums of the warp, then of the CTA (fixed order)
+        if constexpr (kCluster) {  // per-head sums of the warp (fixed order)
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    float v = zv[nt][j];
-                    v += __shfl_xor_sync(0xffffffffu, v, 4);
-                    v += __shfl_xor_sync(0xffffffffu, v, 8);
-                    v += __shfl_xor_sync(0xffffffffu, v, 16);
-                    if (g == 0) z_w[warp * GP + nt * 8 + 2 * qd + j] = v;
-                }
+            for (int nt = 0; nt < NT; ++nt) {
+                float v = zv[nt];
+                v += __shfl_xor_sync(0xffffffffu, v, 1);
+                v += __shfl_xor_sync(0xffffffffu, v, 2);
+                if (qd == 0) z_w[warp * GP + nt * 8 + g] = v;
+            }
+            asm volatile("cp.async.wait_all;" ::: "memory");  // this thread's old scores have landed
         }
         // Partial outputs of this warp, then of the CTA (fixed summation order).
         asm volatile("bar.sync 1, %0;" ::"r"(kConsumerWarps * 32) : "memory");  // the ring is drained
+        if constexpr (kCluster) {  // the CTA's maximum and normaliser, and what a warp's p are scaled by
+            if (tid < GP) {
+                float f[kConsumerWarps], z = 0.f;
+                m_cta[tid] = warp_factors(m_w + tid, f);
+#pragma unroll
+                for (int w = 0; w < kConsumerWarps; ++w) {
+                    f_w[w * GP + tid] = f[w];
+                    z += f[w] * z_w[w * GP + tid];
+                }
+                z_cta[tid] = z;
+            }
+        }
         constexpr int OS = Lay::kOStride;
         float *ow = o_w + warp * GP * OS;
 #pragma unroll
@@ -546,28 +599,27 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
                 ow[(h0 + 1) * OS + d0 + 8] = oacc[i][nt][3];
             }
         asm volatile("bar.sync 1, %0;" ::"r"(kConsumerWarps * 32) : "memory");
-        for (int e = tid; e < GP * D; e += kConsumerWarps * 32) {
-            const int at = (e / D) * OS + e % D;
-            float v = o_w[at];
+        for (int e = tid; e < GP * D / 4; e += kConsumerWarps * 32) {
+            const int h = e / (D / 4), at = h * OS + e % (D / 4) * 4;
+            float f[kConsumerWarps];
+            if constexpr (kCluster) warp_factors(m_w + h, f);
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-            for (int w = 1; w < kConsumerWarps; ++w) v += o_w[w * GP * OS + at];
-            o_cta[at] = v;
-        }
-        if (clustered && tid < GP) {
-            float v = 0.f;
-#pragma unroll
-            for (int w = 0; w < kConsumerWarps; ++w) v += z_w[w * GP + tid];
-            z_cta[tid] = v;
+            for (int w = 0; w < kConsumerWarps; ++w) {
+                const float4 x = *reinterpret_cast<const float4 *>(o_w + w * GP * OS + at);
+                const float s = kCluster ? f[w] : 1.f;
+                v.x += s * x.x, v.y += s * x.y, v.z += s * x.z, v.w += s * x.w;
+            }
+            *reinterpret_cast<float4 *>(o_cta + at) = v;
         }
     }
     if (!ok) raise_status(p.status, VOXZIP_DEV_TIMEOUT);
     ptx::launch_dependents();  // streaming is over: the next launch may begin its prologue
-    __syncthreads();
     // CTA r writes slice r of the G x D outputs: the CTAs' partial outputs summed, normalised.
     constexpr int OS = Lay::kOStride;
     const int o_total = p.G * D;
     __nv_bfloat16 *og = p.out + (act_row * p.Hq + (int64_t)ui.h * p.G) * D;
-    if (clustered) {
+    if constexpr (kCluster) {
         cluster.sync();  // every CTA's m_cta, z_cta, o_cta are final
         // For a cluster of SS CTAs (a power of two), this thread's share of the slice is at most E
         // elements: all their partials from every CTA are requested before the statistics, so the
@@ -604,7 +656,12 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
                 }
                 const float rzv = tid < p.G ? 1.f / z : 0.f;
 #pragma unroll
-                for (int r = 0; r < SS; ++r) fac[r * GP + tid] = mr[r] * rzv;
+                for (int r = 0; r < SS; ++r) {
+                    fac[r * GP + tid] = mr[r] * rzv;
+                    if (r == rank)  // what turns this CTA's kept p (relative to their warp's maximum) into softmax mass
+#pragma unroll
+                        for (int w = 0; w < kConsumerWarps; ++w) f_w[w * GP + tid] *= mr[r] * rzv;
+                }
             }
             __syncthreads();
 #pragma unroll
@@ -631,11 +688,11 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
         // shared memory and global memory.
         asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
         // Eq. 6 for this CTA's tokens: A = gamma * [A, 0] + sum over the group's heads.
-        const float *fs = fac + rank * GP;
         float *sc = p.score + row_base + j0;
         for (int i = tid; i < cnt; i += kThreads) {
             float add = 0.f;
-            const float4 *pr = reinterpret_cast<const float4 *>(lg + i * GP);
+            const float *fs = f_w + (i % kTile) / 16 * GP;  // the warp that took this token
+            const float4 *pr = reinterpret_cast<const float4 *>(lg + lg_row(i) * GP);
 #pragma unroll
             for (int h4 = 0; h4 < GP / 4; ++h4) {
                 const float4 v = pr[h4];
@@ -644,6 +701,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
             if (VOXZIP_IN_RANGE(p.status, j0 + i < p.C)) sc[i] = i == jn ? add : p.gamma * s_old[i] + add;
         }
     } else {
+        __syncthreads();
         for (int i = tid; i < o_total; i += kThreads) {
             const int h = i / D;
             og[i] = __float2bfloat16_rn(o_cta[h * OS + i % D] * fac[h]);
@@ -659,7 +717,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
         }
     }
     // No CTA leaves while a peer may still read its shared memory.
-    if (clustered) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if constexpr (kCluster) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // ---------------------------------------------------------------- host side

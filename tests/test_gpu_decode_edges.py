@@ -1,0 +1,68 @@
+"""The bf16 decode step at the edges of its tiles (64 tokens), of a warp's share of a tile (16) and of
+a CTA's range, over the cluster sizes the planner takes, against the oracle. Some key rows overflow:
+their logits are far below (or -inf in fp32), a whole warp's tokens among them, and weigh nothing."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from gpu_harness import SCORE_ATOL, SCORE_RTOL
+from paper_2608_08569_gb300 import CacheDesc, allocate_cache, voxzip_decode_step, voxzip_get_status
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_08569_gb300 import build
+    build.build_library()
+    oracle.build()
+    voxzip_get_status()
+
+
+@pytest.mark.parametrize("D,Hq,Hkv", [(128, 32, 4), (64, 16, 1), (128, 16, 1)])
+@pytest.mark.parametrize("capacity", [66, 520, 2100])
+@pytest.mark.parametrize("low_rows", [False, True])
+def test_decode_edges(D, Hq, Hkv, capacity, low_rows):
+    edges = [0, 1, 14, 15, 16, 17, 31, 32, 47, 48, 62, 63, 64, 65, 126, 127, 128, 129, 255, 256, 511, 512, 1023, 2047,
+             2049]
+    lens = sorted({min(e, capacity - 1) for e in edges})
+    B, G, dt = len(lens), Hq // Hkv, torch.bfloat16
+    desc = CacheDesc(B, 1, Hq, Hkv, D, capacity, dt)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(capacity + D)
+    c = allocate_cache(desc)
+    for x in ("k", "v"):
+        c[x].normal_(generator=g)
+    c["score"].uniform_(generator=g)
+    c["pos"].copy_(torch.arange(capacity, dtype=torch.int32, device="cuda"))
+    q = torch.randn(1, B, Hq, D, generator=g, device="cuda").to(dt)
+    if low_rows:  # logits of about -1e38 (finite) and below the fp32 range, 16 to 31 whole warps' worth
+        q[..., 0] = 4.0
+        c["k"][:, :, :, 16:32, 0] = -3e38
+        c["k"][:, :, :, 40:52, 0] = -3e38
+        c["k"][:, :, :, 96:128, 0] = -1e37
+    kn, vn = (torch.randn(1, B, Hkv, D, generator=g, device="cuda").to(dt) for _ in range(2))
+    c["len"].copy_(torch.tensor(lens, dtype=torch.int32, device="cuda")[:, None, None].expand(B, 1, Hkv))
+    before = {x: y.clone() for x, y in c.items()}
+    npos = torch.full((B,), 70000, dtype=torch.int32, device="cuda")
+    out = torch.empty_like(q)
+    voxzip_decode_step(desc, 0, 1, q, kn, vn, npos, c["k"], c["v"], c["score"], c["pos"], c["len"], 0.99, out)
+    assert voxzip_get_status() == 0
+    f = lambda t: t.to("cpu", torch.float64).numpy()
+    for b, n in enumerate(lens):
+        for h in range(Hkv):
+            u = oracle.UnitCache.from_rows(capacity, f(before["k"][b, 0, h, :n]), f(before["v"][b, 0, h, :n]),
+                                           before["pos"][b, 0, h, :n].cpu().numpy(), f(before["score"][b, 0, h, :n]))
+            o = oracle.decode_step(u, f(q[0, b, h * G:(h + 1) * G]), f(kn[0, b, h]), f(vn[0, b, h]), 70000, 0.99,
+                                   1 / math.sqrt(D))
+            assert np.abs(f(out[0, b, h * G:(h + 1) * G]) - o).max() <= 2e-2, (n, h)
+            np.testing.assert_allclose(f(c["score"][b, 0, h, :n + 1]), u.score[:n + 1], rtol=SCORE_RTOL,
+                                       atol=SCORE_ATOL)
+            np.testing.assert_array_equal(f(c["k"][b, 0, h, :n + 1]), u.K[:n + 1])
+            assert int(c["len"][b, 0, h]) == n + 1
+            assert torch.equal(c["score"][b, 0, h, n + 1:], before["score"][b, 0, h, n + 1:])

@@ -50,21 +50,6 @@ namespace {
 #ifndef VOXZIP_DECODE_L2_AHEAD
 #define VOXZIP_DECODE_L2_AHEAD 1           // tiles past the ring requested into L2 as each tile issues
 #endif
-#ifndef VOXZIP_DECODE_CTA_FIXED_US
-#define VOXZIP_DECODE_CTA_FIXED_US 5.0     // a CTA's fixed latency: first tiles, exit
-#endif
-#ifndef VOXZIP_DECODE_CLUSTER_FIXED_US
-#define VOXZIP_DECODE_CLUSTER_FIXED_US 0.0  // added by the cluster exchange (S > 1)
-#endif
-#ifndef VOXZIP_DECODE_STAGE_TOKENS_PER_US
-#define VOXZIP_DECODE_STAGE_TOKENS_PER_US 20.0  // one CTA's streaming rate per ring stage in flight
-#endif
-#ifndef VOXZIP_DECODE_SM_TOKENS_PER_US
-#define VOXZIP_DECODE_SM_TOKENS_PER_US 90.0     // one SM's share of HBM bandwidth (~46 GB/s of K+V)
-#endif
-#ifndef VOXZIP_DECODE_GPU_TOKENS_PER_US
-#define VOXZIP_DECODE_GPU_TOKENS_PER_US 12000.0  // the whole GPU near HBM peak (~6.1 TB/s of K+V)
-#endif
 
 constexpr int kConsumerWarps = VOXZIP_DECODE_WARPS;
 constexpr int kThreads = (kConsumerWarps + 1) * 32;
@@ -84,7 +69,7 @@ struct MmaParams {
     int32_t *pos, *len;
     __nv_bfloat16 *out;
     int32_t *status;
-    int32_t B, L, Hq, Hkv, G, C, layer_begin, chunk_cap, n_hint;
+    int32_t B, L, Hq, Hkv, G, C, layer_begin, chunk_cap;
     int64_t rows;  // K / V rows the tensor maps cover (the cache, or the page pools)
     float gamma, scale_log2;
     PageView pv;  // paged instantiations: the pools are k_cache / v_cache
@@ -117,6 +102,34 @@ __device__ __forceinline__ uint32_t swz(int row, int chunk) {  // byte offset in
 // Row of local token i in the logits: within 16 tokens, 8b + 2q + a goes to row 8b + 4a + q, so that
 // phase V's reads (a lane group per q, a and b fixed) take four consecutive rows and no bank twice.
 __device__ __forceinline__ int lg_row(int i) { return (i & ~7) | ((i & 1) << 2) | ((i >> 1) & 3); }
+
+// Tokens per CTA of a unit of n (whole pages when paged).
+template <bool kPaged>
+__device__ __forceinline__ int range_of(int n, int S) {
+    const int c = (n + S - 1) / S;
+    return kPaged ? (c + kTile - 1) / kTile * kTile : c;
+}
+
+// Asks L2 for the first K rows, then V rows, of slots [j0, j0 + cnt) of a cache unit, `budget` rows at
+// most (one warp, all lanes). Hints only: nothing is read but page-table entries, which may be stale.
+template <int D, bool kPaged>
+__device__ __forceinline__ void prefetch_rows(const MmaParams &p, int64_t cache_unit, int j0, int cnt, int budget) {
+    const int lane = threadIdx.x & 31;
+    const int nk = min(cnt, budget), nv = min(cnt, budget - nk);
+    if constexpr (kPaged) {
+        const int32_t *trow = p.pv.table + cache_unit * p.pv.max_pages + j0 / kTile;
+        for (int t = lane; t * kTile < nk; t += 32) {
+            const int64_t row0 = (int64_t)ptx::load_relaxed(trow + t) * kTile;
+            if (row0 < 0 || row0 + kTile > p.rows) continue;  // no page (yet)
+            ptx::prefetch_l2(p.k_cache + row0 * D, (uint32_t)kTile * D * 2);
+            if (t * kTile < nv) ptx::prefetch_l2(p.v_cache + row0 * D, (uint32_t)kTile * D * 2);
+        }
+    } else if (lane == 0) {
+        const int64_t row0 = cache_unit * p.C + j0;
+        if (nk > 0) ptx::prefetch_l2(p.k_cache + row0 * D, (uint32_t)nk * D * 2);
+        if (nv > 0) ptx::prefetch_l2(p.v_cache + row0 * D, (uint32_t)nv * D * 2);
+    }
+}
 
 // kCluster: launched in clusters of S > 1 CTAs (else one CTA holds the whole unit).
 // kPaged: K/V rows live in page pools (see paged.cuh).
@@ -165,34 +178,33 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
         }
         ptx::fence_mbar_init();
     }
-    // While this unit's length is read, pull the first tiles of the range the launch's length hint
-    // predicts into L2 (exact when the unit is as long as the hint; otherwise a few wasted KB).
-    if (!kPaged && warp == kConsumerWarps && lane == 0) {
-        const int est_j0 = rank * ((p.n_hint + S - 1) / S);
-        const int rows = min(kStages * kTile, p.C - est_j0);
-        if (rows > 0) ptx::prefetch_l2(p.k_cache + (row_base + est_j0) * D, (uint32_t)rows * D * 2);
+    // Launched as a programmatic dependent of the previous kernel on the stream, the CTA may start
+    // before that kernel ends. Until then nothing that it writes may be read, but L2 can be asked for
+    // this CTA's first rows while the previous launch drains and HBM idles: K rows, then V rows where
+    // the K range is short, as many as fill the ring (three tiles at least). The unit's length is read
+    // for that atomically, past L1: it may be about to change, so it only aims the prefetch.
+    // Back-to-back launches, against K rows only and the host's length bound: 32 ragged sequences, one
+    // layer each, 21.1 -> 20.2 us; 16 units of 6 400 rows 14.4 -> 13.3; more rows than that gain nothing.
+    int est_j0 = 0, est_cnt = 0;
+    if (warp == kConsumerWarps) {
+        const int seen = min(max(ptx::load_relaxed(p.len + ui.cache_unit), 0), p.C - 1) + 1;
+        const int est_chunk = range_of<kPaged>(seen, S);
+        est_j0 = min(seen, rank * est_chunk);
+        est_cnt = min(seen, est_j0 + est_chunk) - est_j0;
+        prefetch_rows<D, kPaged>(p, ui.cache_unit, est_j0, est_cnt, kTile * (kStages > 3 ? kStages : 3));
     }
     __syncthreads();
-    // Launched as a programmatic dependent of the previous kernel on the stream, the CTA may start
-    // before that kernel ends: everything from here on reads what it wrote (lengths, pages,
-    // cache rows, scores, queries), so wait for its completion. (The prefetch above is a hint.)
+    // Everything from here on reads what the previous kernel wrote (lengths, pages, cache rows,
+    // scores, queries): wait for its completion.
     ptx::grid_dependency_wait();
-    // Paged: before the length is known, the producer reads the page-table entries of the range the
-    // launch's length hint predicts and pulls those tiles into L2 (kept when the prediction holds).
-    int est_j0 = -1, est_tiles = 0;
+    // Paged: before the length is known, the producer reads the page-table entries of the predicted
+    // range (kept when the prediction holds).
+    int est_tiles = 0;
     if constexpr (kPaged) {
         if (warp == kConsumerWarps) {
-            const int est_chunk = ((p.n_hint + S - 1) / S + kTile - 1) / kTile * kTile;
-            est_j0 = rank * est_chunk;
-            est_tiles = max(0, min(est_chunk, p.n_hint - est_j0) + kTile - 1) / kTile;
-            est_tiles = min(est_tiles, p.pv.max_pages - est_j0 / kTile);
+            est_tiles = (est_cnt + kTile - 1) / kTile;
             const int32_t *trow = p.pv.table + ui.cache_unit * p.pv.max_pages + est_j0 / kTile;
-            for (int t = lane; t < est_tiles; t += 32) {
-                const int32_t page = trow[t];
-                tile_rows[t] = page * kTile;
-                if (t < kStages && page >= 0)
-                    ptx::prefetch_l2(p.k_cache + (int64_t)page * kTile * D, (uint32_t)kTile * D * 2);
-            }
+            for (int t = lane; t < est_tiles; t += 32) tile_rows[t] = trow[t] * kTile;
         }
     }
     // The queries do not depend on the length: load them first. Q^T is the B operand:
@@ -229,7 +241,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
             return;
         }
     }
-    const int chunk = kPaged ? ((n + S - 1) / S + kTile - 1) / kTile * kTile : (n + S - 1) / S;
+    const int chunk = range_of<kPaged>(n, S);
     if (chunk > p.chunk_cap) {
         if (rank == 0 && tid == 0) raise_status(p.status, VOXZIP_DEV_LEN_HINT);
         return;
@@ -823,33 +835,35 @@ struct Plan {
     int S, NS, chunk_cap;
 };
 
+// Constants of the planner's time model, fitted to 1 985 timings of forced plans on GB300 (D = 128):
+// launches of 4 to 1 536 units of 60 to 11 520 rows, one layer or all, every S and NS, back to back in a
+// CUDA graph. The plans it picks are 0.7% slower on average than the best of each shape (11% at worst)
+// where the rows come from HBM, and 0.3% (6%) where they stay in L2; the constants that went before
+// (5 us fixed, 20 rows/us a stage, 90 an SM, no cost of sharing an SM) took 4.2% (53%) on the first.
 struct PlanModel {
-    double cta_fixed_us, cluster_fixed_us, stage_tokens_per_us, sm_tokens_per_us, gpu_tokens_per_us;
-    int stage_cap;  // ring stages beyond this add no streaming rate
+    double fixed_us;           // a CTA's prologue and epilogue
+    double shared_us;          // more for each CTA that shares its SM
+    double cluster_us;         // the cluster exchange (S > 1)
+    double cluster16_us;       // more for 16 CTAs, a size that few GPCs hold twice
+    double stage_rows_per_us;  // a CTA's streaming rate per ring stage
+    double cta_rows_per_us;    // what its consumer warps take
+    double sm_rows_per_us;     // what the CTAs of an SM share
+    double last_round;         // how far a part-filled last round costs a whole one
 };
-// A launch whose K and V stream from HBM.
-constexpr PlanModel kPlanModel{VOXZIP_DECODE_CTA_FIXED_US, VOXZIP_DECODE_CLUSTER_FIXED_US,
-                               VOXZIP_DECODE_STAGE_TOKENS_PER_US, VOXZIP_DECODE_SM_TOKENS_PER_US,
-                               VOXZIP_DECODE_GPU_TOKENS_PER_US, 8};
-// A launch whose K and V fit comfortably in L2 (at most VOXZIP_DECODE_L2_RESIDENT_MB): in a decode
-// loop they stay there from step to step. Fitted to back-to-back graph loops on GB300 (10-min and
-// 30-s requests, cluster sizes 1-4, ring depths 2-4): a CTA then consumes ~46 tokens/us whatever
-// its ring depth past three stages, an SM ~120, and a cluster exchange adds ~2.6 us.
-constexpr PlanModel kPlanModelL2{VOXZIP_DECODE_CTA_FIXED_US, 2.6, 46.0 / 3.0, 120.0, 30000.0, 3};
-#ifndef VOXZIP_DECODE_L2_RESIDENT_MB
-#define VOXZIP_DECODE_L2_RESIDENT_MB 64.0
-#endif
+constexpr PlanModel kPlanHbm{4.3, 0.88, 0.2, 0.6, 25.9, 81.0, 163.0, 0.77};
+// A cache that fits comfortably in L2 as a whole: in a decode loop it stays there from step to step.
+constexpr PlanModel kPlanL2{5.0, 0.69, 0.2, 1.4, 28.3, 85.0, 221.0, 0.36};
+constexpr double kL2ResidentBytes = 64.0 * 1048576.0;
 
 // Chooses the cluster size S and ring depth NS with a time model. For each (S, NS) the CTAs hold
 // ceil(nmax/S) tokens (shared memory sized for that, rounded up to 16 tokens); the occupancy API
-// gives how many clusters are resident. Every resident cluster takes ceil(units / clusters) units
-// in turn; a unit costs a CTA's fixed latency (more with a cluster exchange) plus its tokens at one
-// CTA's streaming rate, which grows with the ring stages in flight until the CTAs resident on an SM
-// share its bandwidth; and no launch beats the GPU's streaming rate. A launch small enough to stay
-// in L2 across a decode loop is planned with the L2 constants instead.
-Plan plan(int D, int NT, int units, int nmax, bool paged = false) {
-    const bool l2 = (double)units * nmax * 4.0 * D <= VOXZIP_DECODE_L2_RESIDENT_MB * 1048576.0;
-    const PlanModel &md = l2 ? kPlanModelL2 : kPlanModel;
+// gives how many clusters are resident. Every resident cluster takes its share of the units in turn;
+// a unit costs a CTA's fixed latency (more with a cluster exchange, and with neighbours on its SM)
+// plus its tokens at one CTA's streaming rate, which grows with the ring stages in flight until its
+// consumer warps or the CTAs that share its SM bound it.
+Plan plan(int D, int NT, int units, int nmax, bool paged, bool l2) {
+    const PlanModel &md = l2 ? kPlanL2 : kPlanHbm;
+    const int nmid = max(1, nmax - kTile / 2);  // nmax is a bucket's upper end
     Plan best{0, 3, 0};
     double best_cost = 0.0;
     int sms = 148;
@@ -857,7 +871,6 @@ Plan plan(int D, int NT, int units, int nmax, bool paged = false) {
         int dev = 0;
         if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     }
-    const double total = (double)units * nmax;
     for (int S = 1; S <= kMaxCluster; S <<= 1) {
         int cap = (nmax + S - 1) / S;
         if (S > 1 && cap < kTile / 2) break;
@@ -871,11 +884,13 @@ Plan plan(int D, int NT, int units, int nmax, bool paged = false) {
             const int cl = dispatch(D, NT, ns, [&](auto k) { return max_active_clusters<decltype(k)>(S, sm); });
             if (cl <= 0) continue;
             const double per_sm = fmax(1.0, (double)min(units, cl) * S / sms);  // CTAs sharing an SM
-            const double rate = fmin(md.stage_tokens_per_us * min(ns, md.stage_cap), md.sm_tokens_per_us / per_sm);
-            const double rounds = (double)((units + cl - 1) / cl);
-            const double per_cta = md.cta_fixed_us + (S > 1 ? md.cluster_fixed_us : 0.0) +
-                                   (double)((nmax + S - 1) / S) / rate;
-            const double cost = fmax(rounds * per_cta, total / md.gpu_tokens_per_us);
+            const double rate = fmin(fmin(md.stage_rows_per_us * ns, md.cta_rows_per_us),
+                                     md.sm_rows_per_us * (128.0 / D) / per_sm);  // shorter rows: more of them
+            const double fixed = md.fixed_us + md.shared_us * (per_sm - 1.0) + (S > 1 ? md.cluster_us : 0.0) +
+                                 (S == 16 ? md.cluster16_us : 0.0);
+            const double share = (double)units / cl;
+            const double rounds = share <= 1.0 ? 1.0 : md.last_round * ceil(share) + (1.0 - md.last_round) * share;
+            const double cost = rounds * (fixed + (double)((nmid + S - 1) / S) / rate);
             if (best.S == 0 || cost < best_cost) {
                 best = Plan{S, ns, cap};
                 best_cost = cost;
@@ -908,10 +923,11 @@ cudaError_t launch_impl(const voxzip_cache_desc &d, void *k_base, void *v_base, 
     const int NT = G <= 8 ? 1 : 2;
     const int units = layer_count * d.batch * d.kv_heads;
     const int nmax = (max_len > 0 && max_len < d.capacity) ? max_len : d.capacity;
-    // Plans are cached per (head dim, group tiles, units, length bucket of one tile, layout).
+    const bool l2 = (double)d.batch * d.layers * d.kv_heads * nmax * 4.0 * d.head_dim <= kL2ResidentBytes;
+    // Plans are cached per (head dim, group tiles, units, length bucket of one tile, layout, L2 or HBM).
     struct Entry {
         int D, NT, units, bucket;
-        bool paged;
+        bool paged, l2;
         Plan p;
     };
     thread_local Entry cache[16];
@@ -920,15 +936,15 @@ cudaError_t launch_impl(const voxzip_cache_desc &d, void *k_base, void *v_base, 
     Plan pl{0, 0, 0};
     for (const Entry &e : cache)
         if (e.p.S != 0 && e.D == d.head_dim && e.NT == NT && e.units == units && e.bucket == bucket &&
-            e.paged == paged)
+            e.paged == paged && e.l2 == l2)
             pl = e.p;
     if (pl.S == 0) {
-        pl = plan(d.head_dim, NT, units, bucket * kTile, paged);
+        pl = plan(d.head_dim, NT, units, bucket * kTile, paged, l2);
         if (pl.S == 0) {
             *unsupported = true;
             return cudaSuccess;
         }
-        cache[cache_next] = Entry{d.head_dim, NT, units, bucket, paged, pl};
+        cache[cache_next] = Entry{d.head_dim, NT, units, bucket, paged, l2, pl};
         cache_next = (cache_next + 1) % 16;
     }
     const int S = pl.S;
@@ -962,7 +978,7 @@ cudaError_t launch_impl(const voxzip_cache_desc &d, void *k_base, void *v_base, 
     prm.out = static_cast<__nv_bfloat16 *>(out);
     prm.status = status;
     prm.B = d.batch; prm.L = d.layers; prm.Hq = d.q_heads; prm.Hkv = d.kv_heads; prm.G = G;
-    prm.C = d.capacity; prm.layer_begin = layer_begin; prm.chunk_cap = chunk_cap; prm.n_hint = nmax;
+    prm.C = d.capacity; prm.layer_begin = layer_begin; prm.chunk_cap = chunk_cap;
     prm.rows = rows;
     prm.gamma = gamma;
     prm.pv = pv;

@@ -70,6 +70,7 @@ struct MmaParams {
     __nv_bfloat16 *out;
     int32_t *status;
     int32_t B, L, Hq, Hkv, G, C, layer_begin, chunk_cap;
+    int32_t clusters;  // resident at once
     int64_t rows;  // K / V rows the tensor maps cover (the cache, or the page pools)
     float gamma, scale_log2;
     PageView pv;  // paged instantiations: the pools are k_cache / v_cache
@@ -133,7 +134,11 @@ __device__ __forceinline__ void prefetch_rows(const MmaParams &p, int64_t cache_
 
 // kCluster: launched in clusters of S > 1 CTAs (else one CTA holds the whole unit).
 // kPaged: K/V rows live in page pools (see paged.cuh).
-template <int D, int NT, int kStages, bool kCluster, bool kPaged>
+// kNext: the launch has more clusters than are resident at once, so a CTA's place is taken by a later
+// one; its first rows are requested into L2 while this one finishes (60-min 20x, 768 units in seven
+// rounds: 156 -> 152 us a step). An instantiation of its own: in launches of one round, the test alone
+// cost 1-2%. Without a cluster the CTAs of an SM are not in step, and it gained nothing.
+template <int D, int NT, int kStages, bool kCluster, bool kPaged, bool kNext>
 __global__ void __launch_bounds__(kThreads)
 decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant__ CUtensorMap tmv,
                   const MmaParams p) {
@@ -141,6 +146,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
     constexpr int GP = Lay::kGP;
     constexpr int kHalves = Lay::kHalves;
     constexpr int kKSteps = D / 16;
+    constexpr int kAheadRows = kTile * (kStages > 3 ? kStages : 3);  // rows requested into L2 ahead of the ring
 
     cg::cluster_group cluster = cg::this_cluster();
     const int S = (int)cluster.num_blocks();
@@ -191,7 +197,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
         const int est_chunk = range_of<kPaged>(seen, S);
         est_j0 = min(seen, rank * est_chunk);
         est_cnt = min(seen, est_j0 + est_chunk) - est_j0;
-        prefetch_rows<D, kPaged>(p, ui.cache_unit, est_j0, est_cnt, kTile * (kStages > 3 ? kStages : 3));
+        prefetch_rows<D, kPaged>(p, ui.cache_unit, est_j0, est_cnt, kAheadRows);
     }
     __syncthreads();
     // Everything from here on reads what the previous kernel wrote (lengths, pages, cache rows,
@@ -333,6 +339,17 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
             }
         }
         __syncwarp();  // reconverge the producer warp
+        if constexpr (kNext) {
+            // This CTA's loads are all requested and its epilogue is ahead of it: ask L2 for the first rows
+            // of the cluster that follows on these SMs (blocks start in order).
+            const int next = (int)blockIdx.y + p.clusters;
+            if (next < (int)gridDim.y) {
+                const int64_t cu = unit_of(next, p.B, p.L, p.Hkv, p.layer_begin).cache_unit;
+                const int nn = min(max(p.len[cu], 0), p.C - 1) + 1;
+                const int nchunk = range_of<kPaged>(nn, S), nj0 = min(nn, rank * nchunk);
+                prefetch_rows<D, kPaged>(p, cu, nj0, min(nn, nj0 + nchunk) - nj0, kAheadRows);
+            }
+        }
     } else {
         // ------------------------------------------------------------- consumers
         // Running maximum and normaliser of this thread's logits, per head slot (nt, j).
@@ -739,8 +756,9 @@ struct Tag {
 };
 
 // Calls f(Tag<D, NT, NS>{}) for the runtime shape; the kernel is instantiated for D in {64, 128},
-// NT in {1, 2} (group <= 8 or <= 16) and a ring of NS in {3, 4, 6, 8} stages.
-constexpr int kRingDepths[] = {2, 3, 4, 6, 8};
+// NT in {1, 2} (group <= 8 or <= 16) and a ring of NS in {2, 3, 4, 6} stages
+// (eight never beat six).
+constexpr int kRingDepths[] = {2, 3, 4, 6};
 
 template <int D, int NT, typename F>
 auto dispatch_ns(int NS, F &&f) {
@@ -748,7 +766,6 @@ auto dispatch_ns(int NS, F &&f) {
         case 2: return f(Tag<D, NT, 2>{});
         case 4: return f(Tag<D, NT, 4>{});
         case 6: return f(Tag<D, NT, 6>{});
-        case 8: return f(Tag<D, NT, 8>{});
         default: return f(Tag<D, NT, 3>{});
     }
 }
@@ -761,17 +778,23 @@ auto dispatch(int D, int NT, int NS, F &&f) {
 using KernelFn = void (*)(CUtensorMap, CUtensorMap, MmaParams);
 
 template <typename K>
-KernelFn kernel_for(int S, bool paged = false) {
+KernelFn kernel_for(int S, bool paged, bool next) {
+    if (S == 1)
+        return paged ? decode_mma_kernel<K::D, K::NT, K::NS, false, true, false>
+                     : decode_mma_kernel<K::D, K::NT, K::NS, false, false, false>;
     if (paged)
-        return S > 1 ? decode_mma_kernel<K::D, K::NT, K::NS, true, true> : decode_mma_kernel<K::D, K::NT, K::NS, false, true>;
-    return S > 1 ? decode_mma_kernel<K::D, K::NT, K::NS, true, false> : decode_mma_kernel<K::D, K::NT, K::NS, false, false>;
+        return next ? decode_mma_kernel<K::D, K::NT, K::NS, true, true, true>
+                    : decode_mma_kernel<K::D, K::NT, K::NS, true, true, false>;
+    return next ? decode_mma_kernel<K::D, K::NT, K::NS, true, false, true>
+                : decode_mma_kernel<K::D, K::NT, K::NS, true, false, false>;
 }
 
 template <typename K>
 bool configure() {  // kernel attributes are per function; set once per process
     static bool done = false;
     if (!done) {
-        for (KernelFn kern : {kernel_for<K>(1), kernel_for<K>(2), kernel_for<K>(1, true), kernel_for<K>(2, true)})
+        for (KernelFn kern : {kernel_for<K>(1, false, false), kernel_for<K>(1, true, false), kernel_for<K>(2, false, false),
+                              kernel_for<K>(2, false, true), kernel_for<K>(2, true, false), kernel_for<K>(2, true, true)})
             if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess ||
                 cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
                 return false;
@@ -796,7 +819,7 @@ int max_active_clusters(int S, size_t smem) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel_for<K>(S), &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, kernel_for<K>(S, false, false), &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -806,7 +829,7 @@ int max_active_clusters(int S, size_t smem) {
 template <typename K>
 cudaError_t launch_t(const CUtensorMap &tmk, const CUtensorMap &tmv, const MmaParams &prm, int S, int units,
                      cudaStream_t stream, bool paged) {
-    const KernelFn kern = kernel_for<K>(S, paged);
+    const KernelFn kern = kernel_for<K>(S, paged, units > prm.clusters);
     if (!configure<K>()) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)S, (unsigned)units, 1);
@@ -833,6 +856,7 @@ cudaError_t launch_t(const CUtensorMap &tmk, const CUtensorMap &tmv, const MmaPa
 
 struct Plan {
     int S, NS, chunk_cap;
+    int clusters;  // resident at once
 };
 
 // Constants of the planner's time model, fitted to 1 985 timings of forced plans on GB300 (D = 128):
@@ -864,7 +888,7 @@ constexpr double kL2ResidentBytes = 64.0 * 1048576.0;
 Plan plan(int D, int NT, int units, int nmax, bool paged, bool l2) {
     const PlanModel &md = l2 ? kPlanL2 : kPlanHbm;
     const int nmid = max(1, nmax - kTile / 2);  // nmax is a bucket's upper end
-    Plan best{0, 3, 0};
+    Plan best{0, 3, 0, 0};
     double best_cost = 0.0;
     int sms = 148;
     {
@@ -892,7 +916,7 @@ Plan plan(int D, int NT, int units, int nmax, bool paged, bool l2) {
             const double rounds = share <= 1.0 ? 1.0 : md.last_round * ceil(share) + (1.0 - md.last_round) * share;
             const double cost = rounds * (fixed + (double)((nmid + S - 1) / S) / rate);
             if (best.S == 0 || cost < best_cost) {
-                best = Plan{S, ns, cap};
+                best = Plan{S, ns, cap, cl};
                 best_cost = cost;
             }
         }
@@ -933,7 +957,7 @@ cudaError_t launch_impl(const voxzip_cache_desc &d, void *k_base, void *v_base, 
     thread_local Entry cache[16];
     thread_local int cache_next = 0;
     const int bucket = (nmax + kTile - 1) / kTile;
-    Plan pl{0, 0, 0};
+    Plan pl{0, 0, 0, 0};
     for (const Entry &e : cache)
         if (e.p.S != 0 && e.D == d.head_dim && e.NT == NT && e.units == units && e.bucket == bucket &&
             e.paged == paged && e.l2 == l2)
@@ -979,6 +1003,7 @@ cudaError_t launch_impl(const voxzip_cache_desc &d, void *k_base, void *v_base, 
     prm.status = status;
     prm.B = d.batch; prm.L = d.layers; prm.Hq = d.q_heads; prm.Hkv = d.kv_heads; prm.G = G;
     prm.C = d.capacity; prm.layer_begin = layer_begin; prm.chunk_cap = chunk_cap;
+    prm.clusters = pl.clusters;
     prm.rows = rows;
     prm.gamma = gamma;
     prm.pv = pv;

@@ -16,6 +16,8 @@
 //               pass; pos and score = 0. A persistent grid walks (128-slot chunk, unit) items;
 //               prefill rows in pinned host memory are streamed over the host link by CTAs on
 //               half the SMs;
+//   fuse_ring   the same for rows of at least 256 bytes in device memory, streamed through rings in
+//               shared memory by bulk copies;
 //   fuse_wide   embedding level, any width that is a whole number of 16-byte vectors: one warp per
 //               output row of a sequence, the same arithmetic.
 // Output slots cover the kept tokens of the prompt in order, each a contiguous source range.
@@ -24,6 +26,7 @@
 #include "common.cuh"
 #include "embed.cuh"
 #include "paged.cuh"
+#include "ptx.cuh"
 
 namespace voxzip {
 
@@ -388,6 +391,230 @@ fuse_rows_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
     }
 }
 
+// The same fusion from a ring in shared memory, for prefill rows in device memory. Output slots take
+// consecutive source rows, so the rows of a run of slots are one contiguous block of K and one of V:
+// each warp walks work items (32 slots of a unit) and streams their rows through a ring of its own by
+// 1-D bulk copies, kRingRows rows of K and of V per stage, running ahead into its next item. Rows then
+// come from shared memory in token order, one 16-byte vector of the K or V row per lane, and the sums
+// are fuse_rows_kernel's to the last bit.
+// HBM bounds it. The loads of fuse_rows_kernel wait in registers, four rows at most per warp at half an
+// SM's warps; here 192 KB per SM are in flight whatever the spans. voxzip_anchor_fuse as a whole, bf16,
+// D = 128: 4 x 46 024 tokens, 48 layers (25.5 GB) 4.63 -> 3.87 ms, 0.97 of the measured copy rate; 32
+// ragged sequences of up to 6 256 tokens 2.96 -> 2.43 ms; one of 8 012 tokens 206 -> 189 us (in fp32 344
+// -> 330); a 30-s clip the same 45.5 us. 16 warps: the sums are issue-bound with fewer (12 warps of four
+// stages 4.46 ms, 8 of six 6.05), and two deep stages for 24 warps run dry (4.24).
+template <typename T, int D>
+struct FuseRing {
+    static constexpr int kRowBytes = D * (int)sizeof(T);
+    static constexpr int kWarps = 16;
+    static constexpr int kDepth = 3;
+    static constexpr int kRows = 4096 / (2 * kRowBytes);  // K and V rows of a stage
+    static constexpr int kStageBytes = 2 * kRows * kRowBytes;
+    static constexpr size_t kBytes = (size_t)kWarps * kDepth * (kStageBytes + 8);  // stages, then their mbarriers
+    static constexpr int kSlots = 32;                      // slots per work item, one per lane
+};
+constexpr uint32_t kFuseWaitLimit = 1u << 22;  // polls before an mbarrier wait gives up
+
+__device__ __forceinline__ void bulk_load(void *smem_dst, const void *src, uint32_t bytes, uint64_t *bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     ptx::smem_u32(smem_dst)),
+                 "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(ptx::smem_u32(bar))
+                 : "memory");
+}
+
+template <typename T, int D, bool kPaged>
+__global__ void __launch_bounds__(FuseRing<T, D>::kWarps * 32, 1)
+fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, int32_t anchor_stride,
+                 const T *__restrict__ k_prefill, const T *__restrict__ v_prefill,
+                 const T *__restrict__ anchor_k, const T *__restrict__ anchor_v, FuseWorkspace ws,
+                 T *__restrict__ k_cache, T *__restrict__ v_cache, float *__restrict__ score,
+                 int32_t *__restrict__ pos, int32_t *__restrict__ len, PageView pv) {
+    using FR = FuseRing<T, D>;
+    constexpr int kElems = 16 / (int)sizeof(T);
+    constexpr int kRowVecs = D / kElems;                              // 16-byte vectors of a row
+    constexpr int kPer = 2 * kRowVecs > 32 ? 2 * kRowVecs / 32 : 1;  // vectors per lane: of K, then of V
+    constexpr int kR = FR::kRows, kDepth = FR::kDepth;
+    extern __shared__ __align__(128) uint8_t ring_smem[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint8_t *ring = ring_smem + (size_t)warp * kDepth * FR::kStageBytes;
+    uint64_t *full = reinterpret_cast<uint64_t *>(ring_smem + (size_t)FR::kWarps * kDepth * FR::kStageBytes) + warp * kDepth;
+    if (lane == 0) {
+        for (int i = 0; i < kDepth; ++i) ptx::mbar_init(&full[i], 1);
+        ptx::fence_mbar_init();
+    }
+    __syncwarp();
+
+    const int units = B * L * Hkv;
+    int max_len = 0;
+    for (int bb = 0; bb < B; ++bb) max_len = max(max_len, ws.seq_len[bb]);
+    const int chunks = max(1, (max_len + FR::kSlots - 1) / FR::kSlots);
+    const int64_t items = (int64_t)units * chunks;
+    const int64_t step = (int64_t)gridDim.x * FR::kWarps;
+
+    // A work item: its unit and first slot, and per lane one slot's source range, anchor row and
+    // destination row. Its rows are [r0 of lane 0, r1 of lane n - 1).
+    struct Item {
+        int u, slot0, n;      // n = 0: no item left
+        int32_t r0, r1, a, o;
+    };
+    int64_t cursor = (int64_t)blockIdx.x * FR::kWarps + warp;
+    auto next_item = [&]() {
+        Item it{0, 0, 0, 0, 0, -1, 0};
+        for (; cursor < items && it.n == 0; cursor += step) {
+            const int u = (int)(cursor % units), slot0 = (int)(cursor / units) * FR::kSlots;
+            const int b = u / (L * Hkv);
+            int32_t out_len = ws.seq_len[b];
+            if (kPaged && pv.table[(int64_t)u * pv.max_pages] < 0) out_len = -1;  // the pool could not hold it
+            if (slot0 == 0 && lane == 0) len[u] = out_len < 0 ? 0 : out_len;
+            if (out_len <= slot0) continue;
+            it.u = u;
+            it.slot0 = slot0;
+            it.n = min(FR::kSlots, out_len - slot0);
+            if (lane < it.n) {
+                const int64_t m = (int64_t)b * stride + slot0 + lane;
+                it.r0 = ws.slot_src[m];
+                it.r1 = ws.slot_end[m];
+                it.a = ws.slot_anchor[m];
+                it.o = kPaged ? (int32_t)paged_row(pv, u, slot0 + lane) : slot0 + lane;
+            }
+#ifdef VOXZIP_CHECKED
+            const int32_t lo = __shfl_sync(0xffffffffu, it.r0, 0), hi = __shfl_sync(0xffffffffu, it.r1, it.n - 1);
+            if (!VOXZIP_IN_RANGE(ws.status, lo >= 0 && lo < hi && hi <= stride && slot0 + it.n <= C)) it.n = 0;
+#endif
+        }
+        return it;
+    };
+    Item cur = next_item(), nxt = next_item();
+
+    // Loads: stage after stage, rows of the current item and then of the next one.
+    uint32_t filled = 0, used = 0;     // stages requested; stages read
+    int p_row = 0, p_end = 0, p_u = 0; // what is left of the item being requested
+    int p_at = 0;                      // 0: current item not begun, 1: current, 2: next
+    auto refill = [&]() {
+        while (filled - used < (uint32_t)kDepth) {
+            if (p_row == p_end) {
+                if (p_at == 2) break;
+                const int n = p_at == 0 ? cur.n : nxt.n;
+                if (n == 0) break;
+                p_row = __shfl_sync(0xffffffffu, p_at == 0 ? cur.r0 : nxt.r0, 0);
+                p_end = __shfl_sync(0xffffffffu, p_at == 0 ? cur.r1 : nxt.r1, n - 1);
+                p_u = p_at == 0 ? cur.u : nxt.u;
+                ++p_at;
+                continue;
+            }
+            const int rows = min(kR, p_end - p_row);
+            if (lane == 0) {
+                uint8_t *dst = ring + (filled % kDepth) * FR::kStageBytes;
+                uint64_t *bar = &full[filled % kDepth];
+                const int64_t src = ((int64_t)p_u * stride + p_row) * D;
+                ptx::mbar_arrive_expect_tx(bar, 2u * (uint32_t)rows * FR::kRowBytes);
+                bulk_load(dst, k_prefill + src, (uint32_t)rows * FR::kRowBytes, bar);
+                bulk_load(dst + kR * FR::kRowBytes, v_prefill + src, (uint32_t)rows * FR::kRowBytes, bar);
+            }
+            p_row += rows;
+            ++filled;
+        }
+    };
+    refill();
+
+    // This lane's vectors: of the K row for v < kRowVecs, of the V row after.
+    const bool active = lane < 2 * kRowVecs;
+    bool ok = true;
+    while (cur.n > 0 && ok) {
+        if (lane < cur.n) {
+            pos[(int64_t)cur.u * C + cur.slot0 + lane] = cur.r0;
+            score[(int64_t)cur.u * C + cur.slot0 + lane] = 0.f;
+        }
+        const int64_t out_base = kPaged ? 0 : (int64_t)cur.u * C * D;
+        const int first = __shfl_sync(0xffffffffu, cur.r0, 0);
+        int r = first;       // next row
+        int left = 0;        // rows left in the stage being read
+        const uint8_t *at = ring;
+        for (int k = 0; k < cur.n && ok; ++k) {
+            const int32_t r0 = __shfl_sync(0xffffffffu, cur.r0, k), r1 = __shfl_sync(0xffffffffu, cur.r1, k);
+            const int32_t a_row = __shfl_sync(0xffffffffu, cur.a, k), o_row = __shfl_sync(0xffffffffu, cur.o, k);
+            const bool anchored = anchor_k != nullptr && a_row >= 0 && VOXZIP_IN_RANGE(ws.status, a_row < anchor_stride);
+            uint4 anc[kPer];
+            if (anchored && active) {
+#pragma unroll
+                for (int i = 0; i < kPer; ++i) {
+                    const int v = lane + 32 * i;
+                    anc[i] = *reinterpret_cast<const uint4 *>(
+                        (v < kRowVecs ? anchor_k : anchor_v) + ((int64_t)cur.u * anchor_stride + a_row) * D + v % kRowVecs * kElems);
+                }
+            }
+            float acc[kPer][kElems];
+#pragma unroll
+            for (int i = 0; i < kPer; ++i)
+#pragma unroll
+                for (int e = 0; e < kElems; ++e) acc[i][e] = 0.f;
+            while (r < r1) {
+                if (left == 0) {  // the next stage (the first one of the item, or the one after)
+                    if (r != first) {
+                        __syncwarp();  // every lane has read the stage
+                        ++used;
+                        refill();
+                    }
+                    if (!ptx::mbar_wait_bounded(&full[used % kDepth], (used / kDepth) & 1, kFuseWaitLimit)) ok = false;
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    at = ring + (used % kDepth) * FR::kStageBytes;
+                    left = kR;
+                }
+                const int take = min(left, r1 - r);
+                for (int j = 0; j < take; ++j) {
+#pragma unroll
+                    for (int i = 0; i < kPer; ++i) {
+                        const int v = lane + 32 * i;
+                        if (active)
+                            accumulate16<T>(acc[i], *reinterpret_cast<const uint4 *>(
+                                                        at + (v < kRowVecs ? 0 : kR * FR::kRowBytes) + v % kRowVecs * 16));
+                    }
+                    at += FR::kRowBytes;
+                }
+                left -= take;
+                r += take;
+            }
+            if (!ok) break;
+            if (active) {
+                const float cnt = (float)(r1 - r0);
+                T *out[2] = {k_cache + out_base + (int64_t)o_row * D, v_cache + out_base + (int64_t)o_row * D};
+#pragma unroll
+                for (int i = 0; i < kPer; ++i) {
+                    const int v = lane + 32 * i;
+                    if (r1 - r0 > 1) {
+#pragma unroll
+                        for (int e = 0; e < kElems; ++e) acc[i][e] = __fdiv_rn(acc[i][e], cnt);
+                    }
+                    if (anchored) {
+                        float t[kElems];
+#pragma unroll
+                        for (int e = 0; e < kElems; ++e) t[e] = 0.f;
+                        accumulate16<T>(t, anc[i]);
+#pragma unroll
+                        for (int e = 0; e < kElems; ++e) acc[i][e] = __fadd_rn(acc[i][e], t[e]);
+                    }
+                    *reinterpret_cast<uint4 *>((v < kRowVecs ? out[0] : out[1]) + v % kRowVecs * kElems) = pack16<T>(acc[i]);
+                }
+            }
+        }
+        if (!ok) break;
+        __syncwarp();
+        ++used;  // the item's last stage
+        cur = nxt;
+        if (p_at > 0) --p_at;
+        nxt = next_item();
+        refill();
+    }
+    if (!ok) {  // a wait gave up: let the loads in flight land (bounded) before leaving
+        if (lane == 0) {
+            raise_status(ws.status, VOXZIP_DEV_TIMEOUT);
+            for (uint32_t g = used; g != filled; ++g)
+                (void)ptx::mbar_wait_bounded(&full[g % kDepth], (g / kDepth) & 1, kFuseWaitLimit);
+        }
+    }
+}
+
 template <typename T, int D, bool kPaged = false>
 cudaError_t launch_fuse_rows(const voxzip_cache_desc &d, int32_t stride, int32_t anchor_stride,
                              const void *kp, const void *vp, const void *ak, const void *av,
@@ -414,6 +641,25 @@ cudaError_t launch_fuse_rows(const voxzip_cache_desc &d, int32_t stride, int32_t
     cudaPointerAttributes pa{};
     const bool host_rows = cudaPointerGetAttributes(&pa, kp) == cudaSuccess && pa.type == cudaMemoryTypeHost;
     cudaGetLastError();
+    // Rows of 128 bytes (bf16, D = 64) would leave half of the ring kernel's lanes idle, and rows in host
+    // memory are bound by the link: both keep fuse_rows_kernel.
+    using FR = FuseRing<T, D>;
+    if constexpr (FR::kRowBytes >= 256) if (!host_rows) {
+        static bool configured = false;
+        if (!configured) {
+            const cudaError_t e = cudaFuncSetAttribute(fuse_ring_kernel<T, D, kPaged>,
+                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FR::kBytes);
+            if (e != cudaSuccess) return e;
+            configured = true;
+        }
+        const int64_t ring_items = units * ((stride + FR::kSlots - 1) / FR::kSlots);
+        const unsigned ring_grid = (unsigned)std::max<int64_t>(
+            1, std::min<int64_t>((ring_items + FR::kWarps - 1) / FR::kWarps, sm_count()));
+        fuse_ring_kernel<T, D, kPaged><<<ring_grid, FR::kWarps * 32, FR::kBytes, stream>>>(
+            d.batch, d.layers, d.kv_heads, d.capacity, stride, anchor_stride, (const T *)kp, (const T *)vp,
+            (const T *)ak, (const T *)av, ws, (T *)kc, (T *)vc, score, pos, len, pv);
+        return cudaGetLastError();
+    }
     const int64_t ctas = host_rows ? (VOXZIP_FUSE_HOST_CTAS > 0 ? VOXZIP_FUSE_HOST_CTAS : std::max(1, sm_count() / 2))
                                    : (int64_t)sm_count() * per_sm;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(items, ctas));

@@ -1,0 +1,108 @@
+"""Stage 1 at the edges of its ring kernels: spans shorter than, equal to and many times a ring stage,
+runs of output rows around a work item's, row widths around a team's columns, short, empty and skipped
+sequences beside long ones. Rows, positions, slot maps and lengths are the oracle's bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2608_08569_gb300 import (DEV_BAD_SPANS, CacheDesc, EmbedDesc, allocate_cache, allocate_paged_cache,
+                                    voxzip_anchor_fuse, voxzip_anchor_fuse_paged, voxzip_embed_fuse,
+                                    voxzip_get_status)
+
+pytestmark = pytest.mark.gpu
+
+TEXT = 5   # text tokens before the audio
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_08569_gb300 import build
+    build.build_library()
+    oracle.build()
+    voxzip_get_status()
+
+
+def _sequence(kind, rng):
+    """(in_len, audio_len, spans) with spans as (start, end, groups) in prompt tokens."""
+    if kind == "empty":
+        return 0, 0, []
+    if kind == "bad":            # spans out of order: the sequence is skipped
+        return 60, 40, [(20, 30, 1), (10, 15, 1)]
+    if kind == "one":
+        return TEXT + 1, 1, [(TEXT, TEXT + 1, 3)]
+    if kind == "copied":         # no span: every row is copied
+        return TEXT + 64, 60, []
+    lens = {"small": [1, 2, 3, 4, 5, 7, 8, 9, 15, 16, 17], "long": [33, 1, 200, 64, 31, 96, 1000],
+            "random": list(rng.integers(1, 13, 150))}[kind]
+    t, spans = TEXT, []
+    for l in lens:
+        t += int(rng.integers(0, 3))                      # now and then a gap of background
+        spans.append((t, t + int(l), int(rng.integers(1, 4))))
+        t += int(l)
+    return t + 9, t + 2 - TEXT, spans
+
+
+KINDS = ["small", "empty", "long", "one", "bad", "random", "copied"]
+
+
+def _batch(rng):
+    seqs = [_sequence(k, rng) for k in KINDS]
+    off = np.cumsum([0] + [len(s[2]) for s in seqs])
+    flat = np.array([x for s in seqs for x in s[2]], np.int32).reshape(-1, 3)
+    i32 = lambda x: torch.as_tensor(np.asarray(x), dtype=torch.int32, device="cuda")
+    ints = (i32([s[0] for s in seqs]), i32([min(TEXT, s[0]) for s in seqs]), i32([s[1] for s in seqs]), i32(off),
+            i32(flat[:, 0].copy()), i32(flat[:, 1].copy()), i32(flat[:, 2].copy()))
+    return seqs, ints, max(s[0] for s in seqs) + 3, max(sum(x[2] for x in s[2]) for s in seqs)
+
+
+def _expect(seq, x, anchor, bf16, capacity, keep=True):
+    s, e, g = (np.array([y[i] for y in seq[2]], np.int32) for i in range(3))
+    f = lambda t: t.double().cpu().numpy()
+    return oracle.stage1(f(x[:seq[0]]), seq[0], min(TEXT, seq[0]), seq[1], s, e, g,
+                         anchor=None if anchor is None else f(anchor), cache_is_bf16=bf16, capacity=capacity,
+                         keep_background=keep)
+
+
+@pytest.mark.parametrize("dtype,D", [(torch.bfloat16, 128), (torch.float32, 128), (torch.float32, 64),
+                                     (torch.bfloat16, 64)])
+@pytest.mark.parametrize("anchors", [False, True])
+@pytest.mark.parametrize("paged", [False, True])
+def test_rows(dtype, D, anchors, paged):
+    seqs, ints, stride, A = _batch(np.random.default_rng(7))
+    B, L, H, C = len(seqs), 2, 3, (stride + 63) // 64 * 64
+    desc = CacheDesc(B, L, 2 * H, H, D, C, dtype)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    rnd = lambda n: torch.randn(B, L, H, n, D, generator=g, device="cuda").to(dtype)
+    k, v = rnd(stride), rnd(stride)
+    ak, av = (rnd(A), rnd(A)) if anchors else (None, None)
+    smap = torch.full((B, stride), -7, dtype=torch.int32, device="cuda")
+    if paged:
+        c = allocate_paged_cache(desc, B * L * H * (C // 64 + 1))
+        voxzip_anchor_fuse_paged(desc, c, k, v, *ints, slot_map=smap, anchor_k=ak, anchor_v=av)
+        table = c["page_table"].long().clamp(min=0)
+        kc, vc = (c[x][table].reshape(B, L, H, C, D) for x in ("k_pool", "v_pool"))
+    else:
+        c = allocate_cache(desc)
+        voxzip_anchor_fuse(desc, k, v, *ints, c["k"], c["v"], c["score"], c["pos"], c["len"], slot_map=smap,
+                           anchor_k=ak, anchor_v=av)
+        kc, vc = c["k"], c["v"]
+    assert voxzip_get_status() == DEV_BAD_SPANS
+    for b, seq in enumerate(seqs):
+        for l in range(L):
+            for h in range(H):
+                if KINDS[b] in ("bad", "empty"):
+                    assert int(c["len"][b, l, h]) == 0
+                    continue
+                for x, a, y in ((k, ak, kc), (v, av, vc)):
+                    r = _expect(seq, x[b, l, h], None if a is None else a[b, l, h], dtype == torch.bfloat16, C)
+                    n = r["n"]
+                    assert int(c["len"][b, l, h]) == n
+                    np.testing.assert_array_equal(y[b, l, h, :n].double().cpu().numpy(), r["stored"])
+                np.testing.assert_array_equal(c["pos"][b, l, h, :n].cpu().numpy(), r["pos"])
+                assert not c["score"][b, l, h].any()
+                if not paged:
+                    assert not y[b, l, h, n:].any()

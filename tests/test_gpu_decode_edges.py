@@ -1,6 +1,7 @@
-"""The bf16 decode step at the edges of its tiles (64 tokens), of a warp's share of a tile (16) and of
+"""The decode step at the edges of its tiles (64 tokens), of a warp's share of a tile (16) and of
 a CTA's range, over the cluster sizes the planner takes, against the oracle. Some key rows overflow:
-their logits are far below (or -inf in fp32), a whole warp's tokens among them, and weigh nothing."""
+their logits are far below (or -inf in fp32), a whole warp's tokens among them, and weigh nothing. In
+fp32 every padding of the group, and a range too long for the roomier of the kernel's two layouts."""
 import math
 
 import numpy as np
@@ -24,14 +25,30 @@ def built():
     voxzip_get_status()
 
 
+EDGES = [0, 1, 14, 15, 16, 17, 31, 32, 47, 48, 62, 63, 64, 65, 126, 127, 128, 129, 255, 256, 511, 512, 1023, 2047, 2049]
+
+
 @pytest.mark.parametrize("D,Hq,Hkv", [(128, 32, 4), (64, 16, 1), (128, 16, 1)])
 @pytest.mark.parametrize("capacity", [66, 520, 2100])
 @pytest.mark.parametrize("low_rows", [False, True])
 def test_decode_edges(D, Hq, Hkv, capacity, low_rows):
-    edges = [0, 1, 14, 15, 16, 17, 31, 32, 47, 48, 62, 63, 64, 65, 126, 127, 128, 129, 255, 256, 511, 512, 1023, 2047,
-             2049]
-    lens = sorted({min(e, capacity - 1) for e in edges})
-    B, G, dt = len(lens), Hq // Hkv, torch.bfloat16
+    _check(torch.bfloat16, D, Hq, Hkv, capacity, sorted({min(e, capacity - 1) for e in EDGES}), low_rows, 2e-2)
+
+
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("G", [1, 2, 3, 4, 7, 8, 9, 16])
+@pytest.mark.parametrize("capacity", [66, 2100])
+def test_decode_edges_fp32(D, G, capacity):
+    _check(torch.float32, D, 2 * G, 2, capacity, sorted({min(e, capacity - 1) for e in EDGES}), capacity == 66, 1e-4)
+
+
+@pytest.mark.parametrize("G,n", [(16, 50000), (9, 55000), (1, 300001)])
+def test_decode_long_fp32(G, n):
+    _check(torch.float32, 64, G, 1, n + 5, [n], False, 1e-4)
+
+
+def _check(dt, D, Hq, Hkv, capacity, lens, low_rows, tol):
+    B, G = len(lens), Hq // Hkv
     desc = CacheDesc(B, 1, Hq, Hkv, D, capacity, dt)
     g = torch.Generator(device="cuda")
     g.manual_seed(capacity + D)
@@ -60,7 +77,7 @@ def test_decode_edges(D, Hq, Hkv, capacity, low_rows):
                                            before["pos"][b, 0, h, :n].cpu().numpy(), f(before["score"][b, 0, h, :n]))
             o = oracle.decode_step(u, f(q[0, b, h * G:(h + 1) * G]), f(kn[0, b, h]), f(vn[0, b, h]), 70000, 0.99,
                                    1 / math.sqrt(D))
-            assert np.abs(f(out[0, b, h * G:(h + 1) * G]) - o).max() <= 2e-2, (n, h)
+            assert np.abs(f(out[0, b, h * G:(h + 1) * G]) - o).max() <= tol, (n, h)
             np.testing.assert_allclose(f(c["score"][b, 0, h, :n + 1]), u.score[:n + 1], rtol=SCORE_RTOL,
                                        atol=SCORE_ATOL)
             np.testing.assert_array_equal(f(c["k"][b, 0, h, :n + 1]), u.K[:n + 1])

@@ -669,14 +669,22 @@ cudaError_t launch_fuse_rows(const voxzip_cache_desc &d, int32_t stride, int32_t
     return cudaGetLastError();
 }
 
-constexpr int kWideWarps = 8;
+constexpr int kWideWarps = 8, kWideCtasPerSm = 5;
+constexpr int kWideBatch = 4;  // source rows whose loads a lane has in flight
 
-// Embedding-level fusion: one warp per output row of sequence b; each lane owns 16-byte vectors
-// v and v + 32 of the row (two in flight per source row). The arithmetic is fuse_rows' (fp32 sum
-// in token order, IEEE division by the group size, fp32 anchor add, one rounding).
+// Embedding-level fusion: a warp takes one of `split` column ranges of an output row, 32 16-byte vectors
+// at a time. The arithmetic is fuse_rows' (fp32 sum in token order, IEEE division by the group size,
+// fp32 anchor add, one rounding).
+// Latency and the balance of the warps bound it: an output row has 1 to about 20 source rows, 3.7 on
+// average. So the loads of up to four rows, a tail of fewer included, and of the text row go out
+// together; the next item's metadata is fetched meanwhile; and one vector per lane leaves registers
+// for 40 warps per SM. voxzip_embed_fuse, 4 x 46 024 tokens of 2 048 columns: bf16 228 -> 223 us, fp32
+// 448 -> 364, without the background 184 -> 177. (Two vectors per lane at 24 warps 232; batches of six
+// rows 245, of two 237. Streaming through rings in shared memory, as for K/V, 364: a team of warps
+// shares each row, and the warp that also walks the spans holds back the others.)
 template <typename T>
-__global__ void __launch_bounds__(kWideWarps * 32)
-fuse_wide_kernel(int32_t C, int32_t stride, int32_t D, int32_t text_stride, const T *__restrict__ e_in,
+__global__ void __launch_bounds__(kWideWarps * 32, kWideCtasPerSm)
+fuse_wide_kernel(int32_t C, int32_t stride, int32_t D, int32_t text_stride, int32_t split, const T *__restrict__ e_in,
                  const T *__restrict__ e_text, FuseWorkspace ws, T *__restrict__ e_out, int32_t *__restrict__ pos,
                  int32_t *__restrict__ len) {
     constexpr int kElems = 16 / sizeof(T);
@@ -692,61 +700,55 @@ fuse_wide_kernel(int32_t C, int32_t stride, int32_t D, int32_t text_stride, cons
     const int32_t *src = ws.slot_src + (int64_t)b * stride;
     const int32_t *send = ws.slot_end + (int64_t)b * stride;
     const int32_t *anc = ws.slot_anchor + (int64_t)b * stride;
-    for (int s = blockIdx.x * kWideWarps + warp; s < out_len; s += gridDim.x * kWideWarps) {
-        const int32_t r0 = src[s], r1 = send[s], a_row = anc[s];
+    const int items = out_len * split, step = gridDim.x * kWideWarps;
+    int item = blockIdx.x * kWideWarps + warp;
+    int32_t n0 = 0, n1 = 0, na = -1;
+    if (item < items) {
+        const int s = item / split;
+        n0 = src[s], n1 = send[s], na = anc[s];
+    }
+    for (; item < items; item += step) {
+        const int s = item / split, part = item % split;
+        const int32_t r0 = n0, r1 = n1, a_row = na;
+        if (item + step < items) {
+            const int sn = (item + step) / split;
+            n0 = src[sn], n1 = send[sn], na = anc[sn];
+        }
         if (!VOXZIP_IN_RANGE(ws.status, r0 >= 0 && r0 < r1 && r1 <= stride && s < C &&
                                          (txt == nullptr || a_row < text_stride)))
             continue;
         const float cnt = (float)(r1 - r0);
-        for (int v0 = lane; v0 < vecs; v0 += 64) {
-            const bool two = v0 + 32 < vecs;
-            float acc[2][kElems];
+        const bool anchored = txt != nullptr && a_row >= 0;
+        for (int v = part * 32 + lane; v < vecs; v += split * 32) {
+            uint4 t = make_uint4(0u, 0u, 0u, 0u);
+            if (anchored) t = *reinterpret_cast<const uint4 *>(txt + (int64_t)a_row * D + v * kElems);
+            float acc[kElems];
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
+            for (int e = 0; e < kElems; ++e) acc[e] = 0.f;
+            const uint4 *col = reinterpret_cast<const uint4 *>(in) + ((int64_t)r0 * vecs + v);  // vector v of row r0
+            for (int left = r1 - r0; left > 0; left -= kWideBatch, col += kWideBatch * vecs) {
+                uint4 x[kWideBatch];
 #pragma unroll
-                for (int e = 0; e < kElems; ++e) acc[h][e] = 0.f;
-            const uint4 *col = reinterpret_cast<const uint4 *>(in) + v0;   // vector v0 of row 0
-            const int64_t rstride = vecs;                                    // vectors per row
-            int32_t r = r0;
-            // Four source rows' loads in flight, then their sums in token order.
-            for (; r + 4 <= r1; r += 4) {
-                uint4 x[4][2];
+                for (int i = 0; i < kWideBatch; ++i)
+                    if (i < left) x[i] = __ldcs(col + i * vecs);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    x[i][0] = __ldcs(col + (int64_t)(r + i) * rstride);
-                    x[i][1] = two ? __ldcs(col + (int64_t)(r + i) * rstride + 32) : x[i][0];
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    accumulate16<T>(acc[0], x[i][0]);
-                    accumulate16<T>(acc[1], x[i][1]);
-                }
+                for (int i = 0; i < kWideBatch; ++i)
+                    if (i < left) accumulate16<T>(acc, x[i]);
             }
-            for (; r < r1; ++r) {
-                const uint4 x0 = __ldcs(col + (int64_t)r * rstride);
-                const uint4 x1 = two ? __ldcs(col + (int64_t)r * rstride + 32) : x0;
-                accumulate16<T>(acc[0], x0);
-                accumulate16<T>(acc[1], x1);
+            if (r1 - r0 > 1)
+#pragma unroll
+                for (int e = 0; e < kElems; ++e) acc[e] = __fdiv_rn(acc[e], cnt);
+            if (anchored) {
+                float y[kElems];
+#pragma unroll
+                for (int e = 0; e < kElems; ++e) y[e] = 0.f;
+                accumulate16<T>(y, t);
+#pragma unroll
+                for (int e = 0; e < kElems; ++e) acc[e] = __fadd_rn(acc[e], y[e]);
             }
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (h == 1 && !two) break;
-                const int v = v0 + 32 * h;
-                if (r1 - r0 > 1)
-#pragma unroll
-                    for (int e = 0; e < kElems; ++e) acc[h][e] = __fdiv_rn(acc[h][e], cnt);
-                if (txt != nullptr && a_row >= 0) {
-                    float t[kElems];
-#pragma unroll
-                    for (int e = 0; e < kElems; ++e) t[e] = 0.f;
-                    accumulate16<T>(t, *reinterpret_cast<const uint4 *>(txt + (int64_t)a_row * D + v * kElems));
-#pragma unroll
-                    for (int e = 0; e < kElems; ++e) acc[h][e] = __fadd_rn(acc[h][e], t[e]);
-                }
-                *reinterpret_cast<uint4 *>(out + (int64_t)s * D + v * kElems) = pack16<T>(acc[h]);
-            }
+            *reinterpret_cast<uint4 *>(out + (int64_t)s * D + v * kElems) = pack16<T>(acc);
         }
-        if (lane == 0) pos[(int64_t)b * C + s] = r0;
+        if (lane == 0 && part == 0) pos[(int64_t)b * C + s] = r0;
     }
 }
 
@@ -915,16 +917,20 @@ cudaError_t launch_embed_fuse(int32_t B, int32_t D, int32_t C, bool bf16, const 
                                        in_len, audio_begin, audio_len, span_off, span_start, span_end, span_groups,
                                        ws, slot_map, status, stream);
     if (err != cudaSuccess) return err;
-    // A grid-stride loop over the output rows; about five CTAs of 8 warps per SM in all (the
-    // output has far fewer rows than the prompt stride the slot plan is sized for).
-    const int per_seq = (sm_count() * 5 + B - 1) / B;
-    dim3 grid((unsigned)max(1, min((stride + kWideWarps - 1) / kWideWarps, per_seq)), (unsigned)B);
+    // A grid-stride loop over (output row, column range) items on as many CTAs as are resident. Two
+    // ranges from 96 vectors a row and four from 256: more items balance the warps better, until an item
+    // has too little to load (125 vectors: 1 range 129 us, 2 127, 4 130; 512: 1 385, 2 371, 4 364).
+    const int vecs = D / (bf16 ? 8 : 4);
+    const int split = vecs >= 256 ? 4 : vecs >= 96 ? 2 : 1;
+    const int64_t per_seq = (sm_count() * kWideCtasPerSm + B - 1) / B;
+    const int64_t needed = ((int64_t)stride * split + kWideWarps - 1) / kWideWarps;
+    dim3 grid((unsigned)std::max<int64_t>(1, std::min(needed, per_seq)), (unsigned)B);
     if (bf16)
         fuse_wide_kernel<__nv_bfloat16><<<grid, kWideWarps * 32, 0, stream>>>(
-            C, stride, D, text_stride, (const __nv_bfloat16 *)e_in, (const __nv_bfloat16 *)e_text, ws,
+            C, stride, D, text_stride, split, (const __nv_bfloat16 *)e_in, (const __nv_bfloat16 *)e_text, ws,
             (__nv_bfloat16 *)e_out, pos, len);
     else
-        fuse_wide_kernel<float><<<grid, kWideWarps * 32, 0, stream>>>(C, stride, D, text_stride, (const float *)e_in,
+        fuse_wide_kernel<float><<<grid, kWideWarps * 32, 0, stream>>>(C, stride, D, text_stride, split, (const float *)e_in,
                                                                       (const float *)e_text, ws, (float *)e_out, pos,
                                                                       len);
     return cudaGetLastError();

@@ -106,3 +106,31 @@ def test_rows(dtype, D, anchors, paged):
                 assert not c["score"][b, l, h].any()
                 if not paged:
                     assert not y[b, l, h, n:].any()
+
+
+@pytest.mark.parametrize("dtype,width", [(torch.bfloat16, w) for w in (248, 256, 264, 504, 512, 1000, 1024, 1032, 2048,
+                                                                       2056, 4096, 4608)] +
+                         [(torch.float32, w) for w in (124, 128, 260, 1028, 2048)])
+@pytest.mark.parametrize("text,keep", [(True, True), (False, True), (True, False)])
+def test_embedding_rows(dtype, width, text, keep):
+    seqs, ints, stride, A = _batch(np.random.default_rng(11))
+    B, C = len(seqs), stride
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    e_in = torch.randn(B, stride, width, generator=g, device="cuda").to(dtype)
+    e_text = torch.randn(B, A, width, generator=g, device="cuda").to(dtype) if text else None
+    out = torch.zeros(B, C, width, dtype=dtype, device="cuda")
+    pos = torch.full((B, C), -7, dtype=torch.int32, device="cuda")
+    ln = torch.full((B,), -7, dtype=torch.int32, device="cuda")
+    voxzip_embed_fuse(EmbedDesc(B, width, C, dtype), e_in, *ints, out, pos, ln, e_text=e_text, keep_background=keep)
+    assert voxzip_get_status() == DEV_BAD_SPANS
+    for b, seq in enumerate(seqs):
+        if KINDS[b] in ("bad", "empty"):
+            assert int(ln[b]) == 0 and not out[b].any()
+            continue
+        r = _expect(seq, e_in[b], e_text[b] if text else None, dtype == torch.bfloat16, C, keep)
+        n = r["n"]
+        assert int(ln[b]) == n
+        np.testing.assert_array_equal(out[b, :n].double().cpu().numpy(), r["stored"])
+        np.testing.assert_array_equal(pos[b, :n].cpu().numpy(), r["pos"])
+        assert not out[b, n:].any() and (pos[b, n:] == -7).all()

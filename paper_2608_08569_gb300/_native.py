@@ -56,9 +56,25 @@ class CacheDesc:
     def group(self) -> int:
         return self.q_heads // self.kv_heads
 
+    def __post_init__(self):
+        # What every call needs of the (immutable) descriptor, made once.
+        put, units = object.__setattr__, (self.batch, self.layers, self.kv_heads)
+        put(self, "_units", units)
+        put(self, "_slots", units + (self.capacity,))
+        put(self, "_rows", units + (self.capacity, self.head_dim))
+        try:
+            put(self, "_c", self.c_struct())
+        except (KeyError, TypeError):  # raised again by the call that uses the descriptor
+            put(self, "_c", None)
+
     def c_struct(self) -> _Desc:
         return _Desc(self.batch, self.layers, self.q_heads, self.kv_heads, self.head_dim, self.capacity,
                      _DTYPES[self.dtype])
+
+
+def _c_desc(desc: CacheDesc) -> _Desc:
+    """The binding's own C struct of a descriptor (never handed out: c_struct makes a new one)."""
+    return desc._c if desc._c is not None else desc.c_struct()
 
 
 class _EmbedDesc(ctypes.Structure):
@@ -106,6 +122,8 @@ _EP = ctypes.POINTER(_EmbedDesc)
 def lib() -> ctypes.CDLL:
     """The loaded library; raises if it has not been built (no CPU fallback exists)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -161,17 +179,29 @@ def _check(fn: str, code: int) -> None:
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+# The current stream's handle without a Stream object around it, where torch has the call.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _need(t: torch.Tensor, name: str, dtype: torch.dtype, shape=None, pinned_ok: bool = False) -> None:
     """Checks a tensor argument; `pinned_ok` also accepts page-locked host memory (which the device
     addresses directly under unified addressing)."""
+    # An eager call of a small cache is bound by this binding, not by its kernel: one pass over what
+    # must hold, and the messages only where it does not.
+    if (isinstance(t, torch.Tensor) and t.dtype is dtype and t.is_cuda and t.is_contiguous() and
+            (shape is None or t.shape == shape)):
+        return
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if t.dtype != dtype:
@@ -185,12 +215,9 @@ def _need(t: torch.Tensor, name: str, dtype: torch.dtype, shape=None, pinned_ok:
 
 
 def _check_cache(desc: CacheDesc, k_cache, v_cache, score, pos, len_) -> None:
-    cs = (desc.batch, desc.layers, desc.kv_heads, desc.capacity)
-    _need(k_cache, "k_cache", desc.dtype, cs + (desc.head_dim,))
-    _need(v_cache, "v_cache", desc.dtype, cs + (desc.head_dim,))
-    _need(score, "score", torch.float32, cs)
-    _need(pos, "pos", torch.int32, cs)
-    _need(len_, "len", torch.int32, cs[:3])
+    _need(k_cache, "k_cache", desc.dtype, desc._rows)
+    _need(v_cache, "v_cache", desc.dtype, desc._rows)
+    _check_dense_state(desc, score, pos, len_)
 
 
 def allocate_cache(desc: CacheDesc, device="cuda"):
@@ -235,15 +262,14 @@ def _paged_struct(desc: CacheDesc, pc) -> _Paged:
 
 
 def _check_dense_state(desc: CacheDesc, score, pos, len_) -> None:
-    cs = (desc.batch, desc.layers, desc.kv_heads, desc.capacity)
-    _need(score, "score", torch.float32, cs)
-    _need(pos, "pos", torch.int32, cs)
-    _need(len_, "len", torch.int32, cs[:3])
+    _need(score, "score", torch.float32, desc._slots)
+    _need(pos, "pos", torch.int32, desc._slots)
+    _need(len_, "len", torch.int32, desc._units)
 
 
 def voxzip_paged_init(desc: CacheDesc, pc, stream=None) -> None:
     """Empties every unit of a paged cache (page u for unit u's slot 0, the rest free)."""
-    d, ps = desc.c_struct(), _paged_struct(desc, pc)
+    d, ps = _c_desc(desc), _paged_struct(desc, pc)
     _need(pc["len"], "len", torch.int32, (desc.batch, desc.layers, desc.kv_heads))
     _check("voxzip_paged_init", lib().voxzip_paged_init(ctypes.byref(d), ctypes.byref(ps), _ptr(pc["len"]),
                                                         _stream(stream)))
@@ -277,7 +303,7 @@ def voxzip_anchor_fuse_paged(desc: CacheDesc, pc, k_prefill, v_prefill, in_len, 
         anchor_stride = anchor_k.shape[3]
         _need(anchor_k, "anchor_k", desc.dtype, (B, L, H, anchor_stride, D))
         _need(anchor_v, "anchor_v", desc.dtype, (B, L, H, anchor_stride, D))
-    d, ps = desc.c_struct(), _paged_struct(desc, pc)
+    d, ps = _c_desc(desc), _paged_struct(desc, pc)
     need = int(lib().voxzip_anchor_fuse_paged_workspace_size(ctypes.byref(d), int(stride), int(num_spans)))
     if workspace is None or workspace.numel() < need:
         workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=k_prefill.device)
@@ -299,7 +325,7 @@ def voxzip_decode_step_paged(desc: CacheDesc, pc, layer_begin: int, layer_count:
     _need(out, "out", desc.dtype, (layer_count, B, Hq, D))
     _need(new_pos, "new_pos", torch.int32, (B,))
     _check_dense_state(desc, pc["score"], pc["pos"], pc["len"])
-    d, ps = desc.c_struct(), _paged_struct(desc, pc)
+    d, ps = _c_desc(desc), _paged_struct(desc, pc)
     _check("voxzip_decode_step_paged", lib().voxzip_decode_step_paged(
         ctypes.byref(d), ctypes.byref(ps), int(layer_begin), int(layer_count), _ptr(q), _ptr(k_new), _ptr(v_new),
         _ptr(new_pos), _ptr(pc["score"]), _ptr(pc["pos"]), _ptr(pc["len"]), float(gamma), float(sm_scale),
@@ -322,14 +348,14 @@ def voxzip_evict_paged(desc: CacheDesc, pc, layer_begin: int, layer_count: int, 
         raise ValueError("compaction must be 'ordered' or 'fill'")
     pol = _EvictPolicy(int(sink), float(recent_frac), int(bool(history)), sb, sl,
                        VOXZIP_COMPACT_FILL if compaction == "fill" else VOXZIP_COMPACT_ORDERED)
-    d, ps = desc.c_struct(), _paged_struct(desc, pc)
+    d, ps = _c_desc(desc), _paged_struct(desc, pc)
     _check("voxzip_evict_paged", lib().voxzip_evict_paged(
         ctypes.byref(d), ctypes.byref(ps), int(layer_begin), int(layer_count), _ptr(pc["score"]), _ptr(pc["pos"]),
         _ptr(pc["len"]), _ptr(budget), ctypes.byref(pol), _stream(stream)))
 
 
 def voxzip_anchor_fuse_workspace_size(desc: CacheDesc, prefill_stride: int, num_spans: int) -> int:
-    d = desc.c_struct()
+    d = _c_desc(desc)
     return int(lib().voxzip_anchor_fuse_workspace_size(ctypes.byref(d), int(prefill_stride), int(num_spans)))
 
 
@@ -361,7 +387,7 @@ def voxzip_anchor_fuse(desc: CacheDesc, k_prefill, v_prefill, in_len, audio_begi
     if workspace is None:
         workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=k_cache.device)
     _need(workspace, "workspace", torch.uint8)
-    d = desc.c_struct()
+    d = _c_desc(desc)
     _check("voxzip_anchor_fuse", lib().voxzip_anchor_fuse(
         ctypes.byref(d), _ptr(k_prefill), _ptr(v_prefill), int(stride), _ptr(in_len), _ptr(audio_begin),
         _ptr(audio_len), _ptr(span_off), int(num_spans), _ptr(span_start), _ptr(span_end), _ptr(span_groups),
@@ -459,7 +485,7 @@ def voxzip_anchor_fuse_noalloc(desc: CacheDesc, k_prefill, v_prefill, in_len, au
         anchor_stride = anchor_k.shape[3]
         _need(anchor_k, "anchor_k", desc.dtype, (B, L, H, anchor_stride, D))
         _need(anchor_v, "anchor_v", desc.dtype, (B, L, H, anchor_stride, D))
-    d = desc.c_struct()
+    d = _c_desc(desc)
     _check("voxzip_anchor_fuse_noalloc", lib().voxzip_anchor_fuse_noalloc(
         ctypes.byref(d), _ptr(k_prefill), _ptr(v_prefill), int(stride), _ptr(in_len), _ptr(audio_begin),
         _ptr(audio_len), _ptr(span_off), int(num_spans), _ptr(span_start), _ptr(span_end), _ptr(span_groups),
@@ -478,7 +504,7 @@ def voxzip_decode_step(desc: CacheDesc, layer_begin: int, layer_count: int, q, k
     _need(out, "out", desc.dtype, (layer_count, B, Hq, D))
     _need(new_pos, "new_pos", torch.int32, (B,))
     _check_cache(desc, k_cache, v_cache, score, pos, len_)
-    d = desc.c_struct()
+    d = _c_desc(desc)
     _check("voxzip_decode_step", lib().voxzip_decode_step(
         ctypes.byref(d), int(layer_begin), int(layer_count), _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(new_pos),
         _ptr(k_cache), _ptr(v_cache), _ptr(score), _ptr(pos), _ptr(len_), float(gamma), float(sm_scale),
@@ -490,7 +516,7 @@ def voxzip_evict(desc: CacheDesc, layer_begin: int, layer_count: int, k_cache, v
     """Budgeted eviction (Eq. 7-9) for layers [layer_begin, layer_begin + layer_count)."""
     _check_cache(desc, k_cache, v_cache, score, pos, len_)
     _need(budget, "budget", torch.int32, (desc.batch,))
-    d = desc.c_struct()
+    d = _c_desc(desc)
     _check("voxzip_evict", lib().voxzip_evict(
         ctypes.byref(d), int(layer_begin), int(layer_count), _ptr(k_cache), _ptr(v_cache), _ptr(score), _ptr(pos),
         _ptr(len_), _ptr(budget), int(sink), float(recent_frac), _stream(stream)))
@@ -514,7 +540,7 @@ def voxzip_evict_ex(desc: CacheDesc, layer_begin: int, layer_count: int, k_cache
         raise ValueError("compaction must be 'ordered' or 'fill'")
     pol = _EvictPolicy(int(sink), float(recent_frac), int(bool(history)), sb, sl,
                        VOXZIP_COMPACT_FILL if compaction == "fill" else VOXZIP_COMPACT_ORDERED)
-    d = desc.c_struct()
+    d = _c_desc(desc)
     _check("voxzip_evict_ex", lib().voxzip_evict_ex(
         ctypes.byref(d), int(layer_begin), int(layer_count), _ptr(k_cache), _ptr(v_cache), _ptr(score), _ptr(pos),
         _ptr(len_), _ptr(budget), ctypes.byref(pol), _stream(stream)))

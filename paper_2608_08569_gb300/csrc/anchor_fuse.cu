@@ -400,8 +400,8 @@ fuse_rows_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
 // HBM bounds it. The loads of fuse_rows_kernel wait in registers, four rows at most per warp at half an
 // SM's warps; here 192 KB per SM are in flight whatever the spans. voxzip_anchor_fuse as a whole, bf16,
 // D = 128: 4 x 46 024 tokens, 48 layers (25.5 GB) 4.63 -> 3.87 ms, 0.97 of the measured copy rate; 32
-// ragged sequences of up to 6 256 tokens 2.96 -> 2.43 ms; one of 8 012 tokens 206 -> 189 us (in fp32 344
-// -> 330); a 30-s clip the same 45.5 us. 16 warps: the sums are issue-bound with fewer (12 warps of four
+// ragged sequences of up to 6 256 tokens 2.96 -> 2.43 ms; one of 8 012 tokens 206 -> 180 us (in fp32 344
+// -> 331); a 30-s clip 45.5 -> 38.5. 16 warps: the sums are issue-bound with fewer (12 warps of four
 // stages 4.46 ms, 8 of six 6.05), and two deep stages for 24 warps run dry (4.24).
 template <typename T, int D>
 struct FuseRing {
@@ -411,7 +411,7 @@ struct FuseRing {
     static constexpr int kRows = 4096 / (2 * kRowBytes);  // K and V rows of a stage
     static constexpr int kStageBytes = 2 * kRows * kRowBytes;
     static constexpr size_t kBytes = (size_t)kWarps * kDepth * (kStageBytes + 8);  // stages, then their mbarriers
-    static constexpr int kSlots = 32;                      // slots per work item, one per lane
+    static constexpr int kMaxSlots = 32, kMinSlots = 8;    // slots per work item, one per lane
 };
 constexpr uint32_t kFuseWaitLimit = 1u << 22;  // polls before an mbarrier wait gives up
 
@@ -447,9 +447,14 @@ fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
     const int units = B * L * Hkv;
     int max_len = 0;
     for (int bb = 0; bb < B; ++bb) max_len = max(max_len, ws.seq_len[bb]);
-    const int chunks = max(1, (max_len + FR::kSlots - 1) / FR::kSlots);
-    const int64_t items = (int64_t)units * chunks;
     const int64_t step = (int64_t)gridDim.x * FR::kWarps;
+    // Smaller items where there are few per warp: the last round costs less, and short prompts spread
+    // over more warps (192 units: 8 012 tokens 189 -> 180 us, a 30-s clip 45.7 -> 38.5; the 60-min
+    // request, 180 items of 32 slots per warp, does not gain).
+    int slots = FR::kMaxSlots;
+    while (slots > FR::kMinSlots && (int64_t)units * (max_len / slots) < 12 * step) slots >>= 1;
+    const int chunks = max(1, (max_len + slots - 1) / slots);
+    const int64_t items = (int64_t)units * chunks;
 
     // A work item: its unit and first slot, and per lane one slot's source range, anchor row and
     // destination row. Its rows are [r0 of lane 0, r1 of lane n - 1).
@@ -461,7 +466,7 @@ fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
     auto next_item = [&]() {
         Item it{0, 0, 0, 0, 0, -1, 0};
         for (; cursor < items && it.n == 0; cursor += step) {
-            const int u = (int)(cursor % units), slot0 = (int)(cursor / units) * FR::kSlots;
+            const int u = (int)(cursor % units), slot0 = (int)(cursor / units) * slots;
             const int b = u / (L * Hkv);
             int32_t out_len = ws.seq_len[b];
             if (kPaged && pv.table[(int64_t)u * pv.max_pages] < 0) out_len = -1;  // the pool could not hold it
@@ -469,7 +474,7 @@ fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
             if (out_len <= slot0) continue;
             it.u = u;
             it.slot0 = slot0;
-            it.n = min(FR::kSlots, out_len - slot0);
+            it.n = min(slots, out_len - slot0);
             if (lane < it.n) {
                 const int64_t m = (int64_t)b * stride + slot0 + lane;
                 it.r0 = ws.slot_src[m];
@@ -532,8 +537,9 @@ fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
         const uint8_t *at = ring;
         for (int k = 0; k < cur.n && ok; ++k) {
             const int32_t r0 = __shfl_sync(0xffffffffu, cur.r0, k), r1 = __shfl_sync(0xffffffffu, cur.r1, k);
-            const int32_t a_row = __shfl_sync(0xffffffffu, cur.a, k), o_row = __shfl_sync(0xffffffffu, cur.o, k);
-            const bool anchored = anchor_k != nullptr && a_row >= 0 && VOXZIP_IN_RANGE(ws.status, a_row < anchor_stride);
+            const int32_t a_row = anchor_k != nullptr ? __shfl_sync(0xffffffffu, cur.a, k) : -1;
+            const int32_t o_row = kPaged ? __shfl_sync(0xffffffffu, cur.o, k) : cur.slot0 + k;
+            const bool anchored = a_row >= 0 && VOXZIP_IN_RANGE(ws.status, a_row < anchor_stride);
             uint4 anc[kPer];
             if (anchored && active) {
 #pragma unroll
@@ -577,12 +583,12 @@ fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
             }
             if (!ok) break;
             if (active) {
-                const float cnt = (float)(r1 - r0);
                 T *out[2] = {k_cache + out_base + (int64_t)o_row * D, v_cache + out_base + (int64_t)o_row * D};
 #pragma unroll
                 for (int i = 0; i < kPer; ++i) {
                     const int v = lane + 32 * i;
                     if (r1 - r0 > 1) {
+                        const float cnt = (float)(r1 - r0);
 #pragma unroll
                         for (int e = 0; e < kElems; ++e) acc[i][e] = __fdiv_rn(acc[i][e], cnt);
                     }
@@ -652,7 +658,7 @@ cudaError_t launch_fuse_rows(const voxzip_cache_desc &d, int32_t stride, int32_t
             if (e != cudaSuccess) return e;
             configured = true;
         }
-        const int64_t ring_items = units * ((stride + FR::kSlots - 1) / FR::kSlots);
+        const int64_t ring_items = units * ((stride + FR::kMinSlots - 1) / FR::kMinSlots);
         const unsigned ring_grid = (unsigned)std::max<int64_t>(
             1, std::min<int64_t>((ring_items + FR::kWarps - 1) / FR::kWarps, sm_count()));
         fuse_ring_kernel<T, D, kPaged><<<ring_grid, FR::kWarps * 32, FR::kBytes, stream>>>(

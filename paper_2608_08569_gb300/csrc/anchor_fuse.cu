@@ -25,6 +25,7 @@
 
 #include "common.cuh"
 #include "embed.cuh"
+#include "evict_policy.cuh"
 #include "paged.cuh"
 #include "ptx.cuh"
 
@@ -680,13 +681,12 @@ cudaError_t launch_fuse_rows(const voxzip_cache_desc &d, int32_t stride, int32_t
     // memory are bound by the link: both keep fuse_rows_kernel.
     using FR = FuseRing<T, D>;
     if constexpr (FR::kRowBytes >= 256) if (!host_rows) {
-        static bool configured = false;
-        if (!configured) {
-            const cudaError_t e = cudaFuncSetAttribute(fuse_ring_kernel<T, D, kPaged>,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FR::kBytes);
-            if (e != cudaSuccess) return e;
-            configured = true;
-        }
+        static std::atomic<uint64_t> configured{0};
+        const cudaError_t set = once_per_device(configured, [] {
+            return cudaFuncSetAttribute(fuse_ring_kernel<T, D, kPaged>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)FR::kBytes);
+        });
+        if (set != cudaSuccess) return set;
         const int64_t ring_items = units * ((stride + FR::kMinSlots - 1) / FR::kMinSlots);
         const unsigned ring_grid = (unsigned)std::max<int64_t>(
             1, std::min<int64_t>((ring_items + FR::kWarps - 1) / FR::kWarps, sm_count()));

@@ -371,14 +371,12 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const DecodeParams p) 
 template <typename T, int D, int GP, bool kBig>
 cudaError_t launch_t(const DecodeParams &prm, int S, int units, cudaStream_t stream) {
     auto kern = decode_kernel<T, D, GP, kBig>;
-    static bool configured = false;  // attributes are per function; set once per process
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static std::atomic<uint64_t> configured{0};
+    const cudaError_t set = once_per_device(configured, [&] {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    });
+    if (set != cudaSuccess) return set;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)S, (unsigned)units, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);

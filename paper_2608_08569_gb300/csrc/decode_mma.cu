@@ -35,6 +35,7 @@
 #include <type_traits>
 
 #include "common.cuh"
+#include "evict_policy.cuh"
 #include "paged.cuh"
 #include "ptx.cuh"
 #include "tmap.cuh"
@@ -793,17 +794,18 @@ KernelFn kernel_for(int S, bool paged, bool next) {
 }
 
 template <typename K>
-bool configure() {  // kernel attributes are per function; set once per process
-    static bool done = false;
-    if (!done) {
-        for (KernelFn kern : {kernel_for<K>(1, false, false), kernel_for<K>(1, true, false), kernel_for<K>(2, false, false),
-                              kernel_for<K>(2, false, true), kernel_for<K>(2, true, false), kernel_for<K>(2, true, true)})
-            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem) != cudaSuccess ||
-                cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
-                return false;
-        done = true;
-    }
-    return true;
+bool configure() {
+    static std::atomic<uint64_t> done{0};
+    return once_per_device(done, [] {
+               for (KernelFn kern : {kernel_for<K>(1, false, false), kernel_for<K>(1, true, false),
+                                     kernel_for<K>(2, false, false), kernel_for<K>(2, false, true),
+                                     kernel_for<K>(2, true, false), kernel_for<K>(2, true, true)}) {
+                   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
+                   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+                   if (e != cudaSuccess) return e;
+               }
+               return cudaSuccess;
+           }) == cudaSuccess;
 }
 
 // How many clusters of S CTAs, each with `smem` bytes of shared memory, fit the GPU at once.

@@ -878,10 +878,11 @@ struct PlanModel {
     double cta_rows_per_us;    // what its consumer warps take
     double sm_rows_per_us;     // what the CTAs of an SM share
     double last_round;         // how far a part-filled last round costs a whole one
+    double next_us;            // what a round of clusters saves when the one before asks L2 for its first rows
 };
-constexpr PlanModel kPlanHbm{4.3, 0.88, 0.2, 0.6, 25.9, 81.0, 163.0, 0.77};
+constexpr PlanModel kPlanHbm{4.3, 0.88, 0.2, 0.6, 25.9, 81.0, 163.0, 0.77, 1.2};
 // A cache that fits comfortably in L2 as a whole: in a decode loop it stays there from step to step.
-constexpr PlanModel kPlanL2{5.0, 0.69, 0.2, 1.4, 28.4, 85.0, 221.0, 0.36};  // three stages keep the warps fed
+constexpr PlanModel kPlanL2{5.0, 0.69, 0.2, 1.4, 28.4, 85.0, 221.0, 0.36, 0.0};  // three stages keep the warps fed
 constexpr double kL2ResidentBytes = 64.0 * 1048576.0;
 
 // Chooses the cluster size S and ring depth NS with a time model. For each (S, NS) the CTAs hold
@@ -919,7 +920,8 @@ Plan plan(int D, int NT, int units, int nmax, bool paged, bool l2) {
                                  (S == 16 ? md.cluster16_us : 0.0);
             const double share = (double)units / cl;
             const double rounds = share <= 1.0 ? 1.0 : md.last_round * ceil(share) + (1.0 - md.last_round) * share;
-            const double cost = rounds * (fixed + (double)((nmid + S - 1) / S) / rate);
+            const double cost = rounds * (fixed + (double)((nmid + S - 1) / S) / rate) -
+                                (S > 1 ? (rounds - 1.0) * md.next_us : 0.0);
             if (best.S == 0 || cost < best_cost) {
                 best = Plan{S, ns, cap, cl};
                 best_cost = cost;

@@ -737,7 +737,7 @@ def gpu_arm(args, rank, world, local):
         per_req_ms = ms / args.steps
         roofline_stage1 = {"bound": "hbm", "achieved": round(st1_bytes / (st1_ms / 1000.0) / 1e9, 1), "peak": peak,
                            "unit": "GB/s", "frac": round(st1_bytes / (st1_ms / 1000.0) / 1e9 / peak, 4),
-                           "kernel": "stage 1: span_scan + slot_map + fuse_rows_kernel (timed together)",
+                           "kernel": "stage 1: span_scan + slot_map + fuse_ring_kernel (timed together)",
                            "avg_call_us": round(st1_ms * 1000.0, 1), "alg_bytes_per_call": int(st1_bytes),
                            "stage1_share_of_step": round(st1_ms / per_req_ms, 4)}
 

@@ -19,7 +19,7 @@
 //   fuse_ring   the same for rows of at least 256 bytes in device memory, streamed through rings in
 //               shared memory by bulk copies;
 //   fuse_wide   embedding level, any width that is a whole number of 16-byte vectors: one warp per
-//               output row of a sequence, the same arithmetic.
+//               column range of an output row, the same arithmetic.
 // Output slots cover the kept tokens of the prompt in order, each a contiguous source range.
 #include <algorithm>
 

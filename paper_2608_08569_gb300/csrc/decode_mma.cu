@@ -136,8 +136,8 @@ __device__ __forceinline__ void prefetch_rows(const MmaParams &p, int64_t cache_
 // kCluster: launched in clusters of S > 1 CTAs (else one CTA holds the whole unit).
 // kPaged: K/V rows live in page pools (see paged.cuh).
 // kNext: the launch has more clusters than are resident at once, so a CTA's place is taken by a later
-// one; its first rows are requested into L2 while this one finishes (60-min 20x, 768 units in seven
-// rounds: 156 -> 152 us a step). An instantiation of its own: in launches of one round, the test alone
+// one; its first rows are requested into L2 while this one finishes (60-min 20x, 768 units: 156 -> 152 us a
+// step, and 148 with the 4-CTA clusters in seven rounds that then pay). An instantiation of its own: in launches of one round, the test alone
 // cost 1-2%. Without a cluster the CTAs of an SM are not in step, and it gained nothing.
 template <int D, int NT, int kStages, bool kCluster, bool kPaged, bool kNext>
 __global__ void __launch_bounds__(kThreads)

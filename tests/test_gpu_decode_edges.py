@@ -10,7 +10,8 @@ import torch
 
 import oracle
 from gpu_harness import SCORE_ATOL, SCORE_RTOL
-from paper_2608_08569_gb300 import CacheDesc, allocate_cache, voxzip_decode_step, voxzip_get_status
+from paper_2608_08569_gb300 import (CacheDesc, allocate_cache, allocate_paged_cache, voxzip_decode_step,
+                                    voxzip_decode_step_paged, voxzip_get_status)
 
 pytestmark = pytest.mark.gpu
 
@@ -45,6 +46,52 @@ def test_decode_edges_fp32(D, G, capacity):
 @pytest.mark.parametrize("G,n", [(16, 50000), (9, 55000), (1, 300001)])
 def test_decode_long_fp32(G, n):
     _check(torch.float32, 64, G, 1, n + 5, [n], False, 1e-4)
+
+
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("n", [640, 2333])
+def test_decode_many_units(paged, n):
+    """768 units of ragged lengths: clusters in several rounds, each asking L2 for a later one's rows.
+    Against the same arithmetic in fp64 on the device."""
+    B, L, Hq, H, D, dt = 4, 48, 32, 4, 128, torch.bfloat16
+    C = (n + 64) // 64 * 64
+    desc = CacheDesc(B, L, Hq, H, D, C, dt)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    lens = torch.randint(1, n + 1, (B, L, H), generator=g, device="cuda", dtype=torch.int32)
+    lens[0], lens[1, :, :2], lens[2, 5] = n, n - 63, 0
+    k, v = (torch.randn(B, L, H, C, D, generator=g, device="cuda").to(dt) for _ in range(2))
+    score = torch.rand(B, L, H, C, generator=g, device="cuda")
+    before = score.clone()
+    pos = torch.zeros(B, L, H, C, dtype=torch.int32, device="cuda")
+    q = torch.randn(L, B, Hq, D, generator=g, device="cuda").to(dt)
+    kn, vn = (torch.randn(L, B, H, D, generator=g, device="cuda").to(dt) for _ in range(2))
+    npos, out, ln = torch.full((B,), 9, dtype=torch.int32, device="cuda"), torch.empty_like(q), lens.clone()
+    if paged:
+        pages = B * L * H * (C // 64)
+        order = torch.randperm(pages, generator=g, device="cuda")
+        pc = allocate_paged_cache(desc, pages)
+        pc["k_pool"][order], pc["v_pool"][order] = k.view(pages, 64, D), v.view(pages, 64, D)
+        pc["page_table"].copy_(order.view(pc["page_table"].shape))
+        pc["free_count"].zero_()
+        pc.update(score=score, pos=pos, len=ln)
+        voxzip_decode_step_paged(desc, pc, 0, L, q, kn, vn, npos, 0.99, out, max_len=n + 1)
+    else:
+        voxzip_decode_step(desc, 0, L, q, kn, vn, npos, k, v, score, pos, ln, 0.99, out, max_len=n + 1)
+    assert voxzip_get_status() == 0
+    assert torch.equal(ln, lens + 1)
+    slot = torch.arange(C, device="cuda")
+    for l in range(L):
+        m = lens[:, l].long()
+        at = m[..., None, None].expand(B, H, 1, D)
+        kl = k[:, l].double().scatter(2, at, kn[l].double()[:, :, None])
+        vl = v[:, l].double().scatter(2, at, vn[l].double()[:, :, None])
+        x = q[l].double().view(B, H, Hq // H, D) @ kl.transpose(-1, -2) / math.sqrt(D)
+        p = torch.softmax(x.masked_fill((slot > m[..., None])[:, :, None], -math.inf), -1)
+        assert ((p @ vl).reshape(B, Hq, D) - out[l].double()).abs().max() <= 2e-2
+        old = before[:, l].double().masked_fill(slot == m[..., None], 0.0)
+        want = torch.where(slot <= m[..., None], 0.99 * old + p.sum(2), before[:, l].double())
+        torch.testing.assert_close(score[:, l].double(), want, rtol=SCORE_RTOL, atol=SCORE_ATOL)
 
 
 def _check(dt, D, Hq, Hkv, capacity, lens, low_rows, tol):

@@ -128,6 +128,7 @@ __device__ __forceinline__ void prefetch_rows(const MmaParams &p, int64_t cache_
         }
     } else if (lane == 0) {
         const int64_t row0 = cache_unit * p.C + j0;
+        if (!VOXZIP_IN_RANGE(p.status, row0 >= 0 && row0 + nk <= p.rows)) return;
         if (nk > 0) ptx::prefetch_l2(p.k_cache + row0 * D, (uint32_t)nk * D * 2);
         if (nv > 0) ptx::prefetch_l2(p.v_cache + row0 * D, (uint32_t)nv * D * 2);
     }
@@ -205,13 +206,16 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
     // scores, queries): wait for its completion.
     ptx::grid_dependency_wait();
     // Paged: before the length is known, the producer reads the page-table entries of the predicted
-    // range (kept when the prediction holds).
+    // range (kept when the prediction holds), as many as this CTA's share has room for: the length seen
+    // may be above the launch's bound, in a unit that is about to be skipped or has just been shortened.
     int est_tiles = 0;
     if constexpr (kPaged) {
         if (warp == kConsumerWarps) {
-            est_tiles = (est_cnt + kTile - 1) / kTile;
+            est_tiles = min((est_cnt + kTile - 1) / kTile, p.chunk_cap / kTile);
             const int32_t *trow = p.pv.table + ui.cache_unit * p.pv.max_pages + est_j0 / kTile;
-            for (int t = lane; t < est_tiles; t += 32) tile_rows[t] = trow[t] * kTile;
+            for (int t = lane; t < est_tiles; t += 32)
+                if (VOXZIP_IN_RANGE(p.status, t < p.chunk_cap / kTile && est_j0 / kTile + t < p.pv.max_pages))
+                    tile_rows[t] = trow[t] * kTile;
         }
     }
     // The queries do not depend on the length: load them first. Q^T is the B operand:
@@ -309,7 +313,9 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
         if constexpr (kPaged) {  // the pool row of every tile of the range (j0 is page-aligned)
             if (j0 != est_j0 || ntiles > est_tiles) {
                 const int32_t *trow = p.pv.table + ui.cache_unit * p.pv.max_pages + j0 / kTile;
-                for (int t = lane; t < ntiles; t += 32) tile_rows[t] = trow[t] * kTile;
+                for (int t = lane; t < ntiles; t += 32)
+                    if (VOXZIP_IN_RANGE(p.status, t < p.chunk_cap / kTile && j0 / kTile + t < p.pv.max_pages))
+                        tile_rows[t] = trow[t] * kTile;
             }
             __syncwarp();
         }

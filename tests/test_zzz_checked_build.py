@@ -8,6 +8,7 @@ kernel indexes outside its buffers on any of those cases, and that the checks le
 unchanged.
 """
 import os
+import re
 import subprocess
 import sys
 
@@ -15,7 +16,14 @@ import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 PARITY_FILES = ["tests/test_gpu_parity.py", "tests/test_gpu_paged.py", "tests/test_gpu_policies.py",
-                "tests/test_gpu_embed.py", "tests/test_zzzz_no_alloc.py"]
+                "tests/test_gpu_embed.py", "tests/test_gpu_decode_edges.py", "tests/test_gpu_fuse_ring.py",
+                "tests/test_zzzz_no_alloc.py"]
+
+
+def test_every_parity_file_runs_checked():
+    """Each test file of the kernels is in the list (test_gpu_measure.py times a plain read, no kernel of the path)."""
+    have = {f"tests/{f}" for f in os.listdir(os.path.join(ROOT, "tests")) if re.match(r"test_gpu_\w+\.py$", f)}
+    assert have - {"tests/test_gpu_measure.py"} <= set(PARITY_FILES)
 
 
 @pytest.mark.gpu

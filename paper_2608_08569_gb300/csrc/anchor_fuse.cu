@@ -140,6 +140,8 @@ __host__ __device__ inline size_t carve(const voxzip_cache_desc &d, int32_t stri
 // CTAs start while that one drains, and wait for it (griddepcontrol.wait) before their first access.
 // The gaps between the three launches took 6 us of every call: embeddings of 4 x 60 min 223.3 -> 217.6 us,
 // of 10 min 24.0 -> 20.2; K/V of 10 min, 192 units, 180 -> 174, of a 30-s clip 38.2 -> 31.9.
+// The first kernel may be resident while the caller's last one still writes its inputs, so no kernel takes
+// them as `const __restrict__`, which would allow read-only loads (four 60-min prompts 3 843 us with, 3 844 without).
 template <typename... P, typename... A>
 cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, A... args) {
     cudaLaunchConfig_t cfg = {};
@@ -191,10 +193,9 @@ __device__ int block_excl_scan(int v, int *total) {
 
 __global__ void __launch_bounds__(kScanThreads)
 span_scan_kernel(int32_t B, int32_t stride, int32_t capacity, int32_t num_spans, int32_t anchor_stride,
-                 bool has_anchor, bool keep_bg, const int32_t *__restrict__ in_len, const int32_t *__restrict__ audio_begin,
-                 const int32_t *__restrict__ audio_len, const int32_t *__restrict__ span_off,
-                 const int32_t *__restrict__ span_start, const int32_t *__restrict__ span_end,
-                 const int32_t *__restrict__ span_groups, FuseWorkspace ws, int32_t *status) {
+                 bool has_anchor, bool keep_bg, const int32_t *in_len, const int32_t *audio_begin,
+                 const int32_t *audio_len, const int32_t *span_off, const int32_t *span_start, const int32_t *span_end,
+                 const int32_t *span_groups, FuseWorkspace ws, int32_t *status) {
     ptx::grid_dependency_wait();
     const int b = blockIdx.x;
     __shared__ int bad;
@@ -256,11 +257,9 @@ span_scan_kernel(int32_t B, int32_t stride, int32_t capacity, int32_t num_spans,
 }
 
 __global__ void __launch_bounds__(kMapThreads)
-slot_map_kernel(int32_t stride, bool keep_bg, const int32_t *__restrict__ in_len,
-                const int32_t *__restrict__ audio_begin, const int32_t *__restrict__ audio_len,
-                const int32_t *__restrict__ span_off, const int32_t *__restrict__ span_start,
-                const int32_t *__restrict__ span_end, const int32_t *__restrict__ span_groups, FuseWorkspace ws,
-                int32_t *__restrict__ slot_map) {
+slot_map_kernel(int32_t stride, bool keep_bg, const int32_t *in_len, const int32_t *audio_begin,
+                const int32_t *audio_len, const int32_t *span_off, const int32_t *span_start, const int32_t *span_end,
+                const int32_t *span_groups, FuseWorkspace ws, int32_t *__restrict__ slot_map) {
     ptx::grid_dependency_wait();
     const int b = blockIdx.y;
     const int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -318,8 +317,7 @@ slot_map_kernel(int32_t stride, bool keep_bg, const int32_t *__restrict__ in_len
 template <typename T, int D, bool kPaged>
 __global__ void __launch_bounds__(kFuseWarps * 32, 4)
 fuse_rows_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, int32_t anchor_stride,
-                 const T *__restrict__ k_prefill, const T *__restrict__ v_prefill,
-                 const T *__restrict__ anchor_k, const T *__restrict__ anchor_v, FuseWorkspace ws,
+                 const T *k_prefill, const T *v_prefill, const T *anchor_k, const T *anchor_v, FuseWorkspace ws,
                  T *__restrict__ k_cache, T *__restrict__ v_cache, float *__restrict__ score,
                  int32_t *__restrict__ pos, int32_t *__restrict__ len, PageView pv) {
     constexpr int kElems = 16 / (int)sizeof(T);  // each lane owns one 16-byte vector of a row
@@ -454,8 +452,7 @@ __device__ __forceinline__ void bulk_load(void *smem_dst, const void *src, uint3
 template <typename T, int D, bool kPaged>
 __global__ void __launch_bounds__(FuseRing<T, D>::kWarps * 32, 1)
 fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, int32_t anchor_stride,
-                 const T *__restrict__ k_prefill, const T *__restrict__ v_prefill,
-                 const T *__restrict__ anchor_k, const T *__restrict__ anchor_v, FuseWorkspace ws,
+                 const T *k_prefill, const T *v_prefill, const T *anchor_k, const T *anchor_v, FuseWorkspace ws,
                  T *__restrict__ k_cache, T *__restrict__ v_cache, float *__restrict__ score,
                  int32_t *__restrict__ pos, int32_t *__restrict__ len, PageView pv) {
     using FR = FuseRing<T, D>;
@@ -717,8 +714,8 @@ constexpr int kWideBatch = 4;  // source rows whose loads a lane has in flight
 // shares each row, and the warp that also walks the spans holds back the others.)
 template <typename T>
 __global__ void __launch_bounds__(kWideWarps * 32, kWideCtasPerSm)
-fuse_wide_kernel(int32_t C, int32_t stride, int32_t D, int32_t text_stride, int32_t split, const T *__restrict__ e_in,
-                 const T *__restrict__ e_text, FuseWorkspace ws, T *__restrict__ e_out, int32_t *__restrict__ pos,
+fuse_wide_kernel(int32_t C, int32_t stride, int32_t D, int32_t text_stride, int32_t split, const T *e_in,
+                 const T *e_text, FuseWorkspace ws, T *__restrict__ e_out, int32_t *__restrict__ pos,
                  int32_t *__restrict__ len) {
     constexpr int kElems = 16 / sizeof(T);
     ptx::grid_dependency_wait();

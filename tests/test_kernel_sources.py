@@ -1,0 +1,22 @@
+"""Rules that the CUDA sources keep and that no run can show: what they forbid goes wrong on another
+machine, with another compiler or under another caller's timing."""
+import glob
+import os
+import re
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SOURCES = {os.path.basename(p): open(p).read()
+           for p in sorted(glob.glob(os.path.join(ROOT, "paper_2608_08569_gb300", "csrc", "*.cu*")))}
+KERNELS = [(f, m.group(1), m.group(2)) for f, s in SOURCES.items()
+           for m in re.finditer(r"__global__\s+void\s+(?:__launch_bounds__\([^{;]*?\)\s+)?(\w+)\s*\(([^{;]*?)\)\s*\{", s)]
+
+
+def test_every_kernel_is_found():
+    assert sum(len(re.findall(r"__global__", s)) for s in SOURCES.values()) == len(KERNELS) >= 10
+
+
+def test_no_kernel_promises_that_its_inputs_do_not_change():
+    """A programmatic dependent is resident while the kernel before it still writes: a pointer to constant
+    data marked __restrict__ would allow read-only loads, which such writes must not meet."""
+    bad = [(f, k, p) for f, k, params in KERNELS for p in re.findall(r"const [^,]*__restrict__ \w+", params)]
+    assert not bad, bad

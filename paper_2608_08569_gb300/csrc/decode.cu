@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const DecodeParams p) 
     }
     // Done reading the peers' shared memory (every value has been used above); the score update touches
     // this CTA's own only.
-    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    ptx::cluster_arrive_relaxed();
     // Eq. 6: A = gamma * [A, 0] + sum over the group's heads of the softmax.
     for (int i = tid; i < cnt; i += kThreads) {
         float add = 0.f;
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const DecodeParams p) 
     }
     if (rank == 0 && tid == 0) p.len[ui.cache_unit] = n;
     // No CTA leaves while others may still read its shared memory.
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    ptx::cluster_wait();
 }
 
 template <typename T, int D, int GP, bool kBig>

@@ -354,8 +354,8 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
                 }
             }
         }
-        __syncwarp();  // reconverge the producer warp
         if constexpr (kNext) {
+            __syncwarp();
             // This CTA's loads are all requested and its epilogue is ahead of it: ask L2 for the first rows
             // of the cluster that follows on these SMs (blocks start in order).
             const int next = (int)blockIdx.y + p.clusters;
@@ -366,6 +366,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
                 prefetch_rows<D, kPaged>(p, cu, nj0, min(nn, nj0 + nchunk) - nj0, kAheadRows);
             }
         }
+        __syncwarp();  // reconverge the producer warp before the barriers of the epilogue
     } else {
         // ------------------------------------------------------------- consumers
         // Running maximum and normaliser of this thread's logits, per head slot (nt, j).
@@ -725,7 +726,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
         // they may leave once all have said so. The arrive orders nothing else, so it is relaxed and
         // does not wait for the output stores. The score update below touches only this CTA's own
         // shared memory and global memory.
-        asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+        ptx::cluster_arrive_relaxed();
         // Eq. 6 for this CTA's tokens: A = gamma * [A, 0] + sum over the group's heads.
         float *sc = p.score + row_base + j0;
         for (int i = tid; i < cnt; i += kThreads) {
@@ -756,7 +757,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
         }
     }
     // No CTA leaves while a peer may still read its shared memory.
-    if constexpr (kCluster) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if constexpr (kCluster) ptx::cluster_wait();
 }
 
 // ---------------------------------------------------------------- host side

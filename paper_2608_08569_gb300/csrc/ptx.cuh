@@ -60,6 +60,18 @@ __device__ __forceinline__ int32_t load_relaxed(const int32_t *p) {
     return v;
 }
 
+// ---------------------------------------------------------------- cluster barrier
+// The two halves of a cluster barrier, for warps whose lanes may have parted: the aligned forms want every
+// lane of a warp at the same instruction. The arrive orders no memory access.
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- TMA
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap *map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");

@@ -20,3 +20,13 @@ def test_no_kernel_promises_that_its_inputs_do_not_change():
     data marked __restrict__ would allow read-only loads, which such writes must not meet."""
     bad = [(f, k, p) for f, k, params in KERNELS for p in re.findall(r"const [^,]*__restrict__ \w+", params)]
     assert not bad, bad
+
+
+def test_aligned_cluster_barriers_follow_a_reconvergence():
+    """The aligned forms of the cluster barrier want all lanes of a warp together. They stand in one place
+    each, right after a __syncwarp()."""
+    for f, s in SOURCES.items():
+        lines = [x.strip() for x in s.splitlines()]
+        for i, x in enumerate(lines):
+            if re.search(r"barrier\.cluster\.\S*aligned", x):
+                assert f == "ptx.cuh" and lines[i - 1] == "__syncwarp();", (f, i + 1)

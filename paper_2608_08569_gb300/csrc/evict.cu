@@ -757,15 +757,13 @@ cudaError_t launch_t(const EvictParams &prm, int units, bool fill, cudaStream_t 
     void (*kern)(EvictParams) = fill ? (fill_wide ? evict_fill_kernel<T, D, kPaged, kThreads>
                                                   : evict_fill_kernel<T, D, kPaged, 192>)
                                      : (wide ? evict_kernel<T, D, kPaged, true> : evict_kernel<T, D, kPaged, false>);
-    if (wide) {  // above the default 48 KB of dynamic shared memory: opt in once
-        static bool configured = false;
-        if (!configured) {
-            const cudaError_t e = cudaFuncSetAttribute(evict_kernel<T, D, kPaged, true>,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       (int)BulkRing<T, D>::kBytes);
-            if (e != cudaSuccess) return e;
-            configured = true;
-        }
+    if (wide) {  // above the default 48 KB of dynamic shared memory: opt in
+        static std::atomic<uint64_t> configured{0};
+        const cudaError_t set = once_per_device(configured, [] {
+            return cudaFuncSetAttribute(evict_kernel<T, D, kPaged, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)BulkRing<T, D>::kBytes);
+        });
+        if (set != cudaSuccess) return set;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)units, 1, 1);

@@ -30,3 +30,12 @@ def test_aligned_cluster_barriers_follow_a_reconvergence():
         for i, x in enumerate(lines):
             if re.search(r"barrier\.cluster\.\S*aligned", x):
                 assert f == "ptx.cuh" and lines[i - 1] == "__syncwarp();", (f, i + 1)
+
+
+def test_kernel_attributes_are_set_per_device():
+    """An attribute belongs to a function on a device: a flag of the process would leave a second GPU without
+    it (and is a race between host threads). Every setting is inside once_per_device."""
+    for f, s in SOURCES.items():
+        for m in re.finditer(r"cudaFuncSetAttribute\(", s):
+            assert "once_per_device(" in s[max(0, m.start() - 800):m.start()], (f, s.count("\n", 0, m.start()) + 1)
+        assert not re.search(r"static bool \w+", s), f

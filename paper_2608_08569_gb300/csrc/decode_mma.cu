@@ -962,18 +962,22 @@ cudaError_t launch_impl(const voxzip_cache_desc &d, void *k_base, void *v_base, 
     const int units = layer_count * d.batch * d.kv_heads;
     const int nmax = (max_len > 0 && max_len < d.capacity) ? max_len : d.capacity;
     const bool l2 = (double)d.batch * d.layers * d.kv_heads * nmax * 4.0 * d.head_dim <= kL2ResidentBytes;
-    // Plans are cached per (head dim, group tiles, units, length bucket of one tile, layout, L2 or HBM).
+    // Plans are cached per (device, head dim, group tiles, units, length bucket of one tile, layout, L2 or
+    // HBM): how many clusters are resident is the device's.
     struct Entry {
-        int D, NT, units, bucket;
+        int device, D, NT, units, bucket;
         bool paged, l2;
         Plan p;
     };
     thread_local Entry cache[16];
     thread_local int cache_next = 0;
     const int bucket = (nmax + kTile - 1) / kTile;
+    int device = 0;
+    const cudaError_t got = cudaGetDevice(&device);
+    if (got != cudaSuccess) return got;
     Plan pl{0, 0, 0, 0};
     for (const Entry &e : cache)
-        if (e.p.S != 0 && e.D == d.head_dim && e.NT == NT && e.units == units && e.bucket == bucket &&
+        if (e.p.S != 0 && e.device == device && e.D == d.head_dim && e.NT == NT && e.units == units && e.bucket == bucket &&
             e.paged == paged && e.l2 == l2)
             pl = e.p;
     if (pl.S == 0) {
@@ -982,7 +986,7 @@ cudaError_t launch_impl(const voxzip_cache_desc &d, void *k_base, void *v_base, 
             *unsupported = true;
             return cudaSuccess;
         }
-        cache[cache_next] = Entry{d.head_dim, NT, units, bucket, paged, l2, pl};
+        cache[cache_next] = Entry{device, d.head_dim, NT, units, bucket, paged, l2, pl};
         cache_next = (cache_next + 1) % 16;
     }
     const int S = pl.S;

@@ -39,3 +39,9 @@ def test_kernel_attributes_are_set_per_device():
         for m in re.finditer(r"cudaFuncSetAttribute\(", s):
             assert "once_per_device(" in s[max(0, m.start() - 800):m.start()], (f, s.count("\n", 0, m.start()) + 1)
         assert not re.search(r"static bool \w+", s), f
+
+
+def test_decode_plans_are_kept_per_device():
+    """A plan's cluster size and how many clusters are resident come from the device's occupancy."""
+    s = SOURCES["decode_mma.cu"]
+    assert re.search(r"struct Entry \{\s*int device\b", s) and "e.device == device" in s

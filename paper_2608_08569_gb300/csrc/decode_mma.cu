@@ -357,11 +357,12 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
         if constexpr (kNext) {
             __syncwarp();
             // This CTA's loads are all requested and its epilogue is ahead of it: ask L2 for the first rows
-            // of the cluster that follows on these SMs (blocks start in order).
+            // of the cluster that follows on these SMs (blocks start in order). It may have started already, and
+            // a short one have stored its new length, so the length is read atomically; it only aims hints.
             const int next = (int)blockIdx.y + p.clusters;
             if (next < (int)gridDim.y) {
                 const int64_t cu = unit_of(next, p.B, p.L, p.Hkv, p.layer_begin).cache_unit;
-                const int nn = min(max(p.len[cu], 0), p.C - 1) + 1;
+                const int nn = min(max(ptx::load_relaxed(p.len + cu), 0), p.C - 1) + 1;
                 const int nchunk = range_of<kPaged>(nn, S), nj0 = min(nn, rank * nchunk);
                 prefetch_rows<D, kPaged>(p, cu, nj0, min(nn, nj0 + nchunk) - nj0, kAheadRows);
             }

@@ -45,3 +45,8 @@ def test_decode_plans_are_kept_per_device():
     """A plan's cluster size and how many clusters are resident come from the device's occupancy."""
     s = SOURCES["decode_mma.cu"]
     assert re.search(r"struct Entry \{\s*int device\b", s) and "e.device == device" in s
+
+
+def test_another_units_length_is_read_atomically():
+    """The cluster of a later unit may run beside this one and store that unit's length."""
+    assert not re.findall(r"p\.len\[(?!ui\.cache_unit\])", SOURCES["decode_mma.cu"])

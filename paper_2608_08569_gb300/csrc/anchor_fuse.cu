@@ -8,7 +8,8 @@
 //               background tokens before the span (dropped in the "Partial" configuration);
 //   slot_map    one thread per prompt token: the output slot of the token (Eq. 4 grouping with
 //               group j = [floor(j*l/g), floor((j+1)*l/g)), Eq. 5 chronological order); the first
-//               token of each slot records the slot's source range and anchor row;
+//               token of each slot records the slot's source range and anchor row; the sequence's
+//               first CTA stores the length of its units (0 when the sequence is skipped);
 //   fuse_rows   K/V level, head_dim 64 or 128: one warp-slice per output slot of every (layer,
 //               kv-head) unit (a lane owns one 16-byte vector of the row; four source rows in
 //               flight): the fp32 mean of the slot's source rows (a copy when the range has one
@@ -259,11 +260,14 @@ span_scan_kernel(int32_t B, int32_t stride, int32_t capacity, int32_t num_spans,
 __global__ void __launch_bounds__(kMapThreads)
 slot_map_kernel(int32_t stride, bool keep_bg, const int32_t *in_len, const int32_t *audio_begin,
                 const int32_t *audio_len, const int32_t *span_off, const int32_t *span_start, const int32_t *span_end,
-                const int32_t *span_groups, FuseWorkspace ws, int32_t *__restrict__ slot_map) {
+                const int32_t *span_groups, FuseWorkspace ws, int32_t *len, int32_t units_per_seq,
+                int32_t *__restrict__ slot_map) {
     ptx::grid_dependency_wait();
     const int b = blockIdx.y;
     const int32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     const int32_t out_len = ws.seq_len[b];
+    if (blockIdx.x == 0)
+        for (int i = threadIdx.x; i < units_per_seq; i += blockDim.x) len[(int64_t)b * units_per_seq + i] = max(out_len, 0);
     const int32_t n_in = in_len[b];
     if (out_len < 0 || t >= n_in) return;
     const int32_t s0 = span_off[b], s1 = span_off[b + 1];
@@ -319,7 +323,7 @@ __global__ void __launch_bounds__(kFuseWarps * 32, 4)
 fuse_rows_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, int32_t anchor_stride,
                  const T *k_prefill, const T *v_prefill, const T *anchor_k, const T *anchor_v, FuseWorkspace ws,
                  T *__restrict__ k_cache, T *__restrict__ v_cache, float *__restrict__ score,
-                 int32_t *__restrict__ pos, int32_t *__restrict__ len, PageView pv) {
+                 int32_t *__restrict__ pos, PageView pv) {
     constexpr int kElems = 16 / (int)sizeof(T);  // each lane owns one 16-byte vector of a row
     constexpr int kLanesPerRow = D / kElems;
     constexpr int kRowsPerWarp = 32 / kLanesPerRow;
@@ -339,7 +343,6 @@ fuse_rows_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
         const int b = u / (L * Hkv);
         int32_t out_len = ws.seq_len[b];
         if (kPaged && pv.table[(int64_t)u * pv.max_pages] < 0) out_len = -1;  // the pool could not hold it
-        if (chunk == 0 && threadIdx.x == 0) len[u] = out_len < 0 ? 0 : out_len;
         if (out_len <= chunk * kSlotsPerPass) continue;
         const int64_t in_base = (int64_t)u * stride * D;
         const int64_t out_base = kPaged ? 0 : (int64_t)u * C * D;
@@ -441,6 +444,9 @@ struct FuseRing {
     static constexpr int kMaxSlots = 32, kMinSlots = 8;    // slots per work item, one per lane
 };
 constexpr uint32_t kFuseWaitLimit = 1u << 22;  // polls before an mbarrier wait gives up
+#ifndef VOXZIP_FUSE_WAIT_LIMIT
+#define VOXZIP_FUSE_WAIT_LIMIT kFuseWaitLimit  // of a wait for rows (0 in a test's build: every wait gives up)
+#endif
 
 __device__ __forceinline__ void bulk_load(void *smem_dst, const void *src, uint32_t bytes, uint64_t *bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
@@ -497,7 +503,6 @@ fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
             const int b = u / (L * Hkv);
             int32_t out_len = ws.seq_len[b];
             if (kPaged && pv.table[(int64_t)u * pv.max_pages] < 0) out_len = -1;  // the pool could not hold it
-            if (slot0 == 0 && lane == 0) len[u] = out_len < 0 ? 0 : out_len;
             if (out_len <= slot0) continue;
             it.u = u;
             it.slot0 = slot0;
@@ -588,9 +593,13 @@ fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
                         ++used;
                         refill();
                     }
-                    if (!ptx::mbar_wait_bounded(&full[used % kDepth], (used / kDepth) & 1, kFuseWaitLimit)) ok = false;
+                    if (!ptx::mbar_wait_bounded(&full[used % kDepth], (used / kDepth) & 1, VOXZIP_FUSE_WAIT_LIMIT)) ok = false;
                     ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) break;
+                    if (!ok) {  // no unit of the call is whole: all become empty (slot_map has stored their lengths)
+#pragma unroll 1
+                        for (int u = lane; u < units; u += 32) len[u] = 0;
+                        break;
+                    }
                     at = ring + (used % kDepth) * FR::kStageBytes;
                     left = kR;
                 }
@@ -696,7 +705,7 @@ cudaError_t launch_fuse_rows(const voxzip_cache_desc &d, int32_t stride, int32_t
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(items, ctas));
     return launch_dependent(fuse_rows_kernel<T, D, kPaged>, dim3(grid), kFuseWarps * 32, 0, stream, d.batch, d.layers,
                             d.kv_heads, d.capacity, stride, anchor_stride, (const T *)kp, (const T *)vp, (const T *)ak,
-                            (const T *)av, ws, (T *)kc, (T *)vc, score, pos, len, pv);
+                            (const T *)av, ws, (T *)kc, (T *)vc, score, pos, pv);
 }
 
 constexpr int kWideWarps = 8, kWideCtasPerSm = 5;
@@ -715,13 +724,11 @@ constexpr int kWideBatch = 4;  // source rows whose loads a lane has in flight
 template <typename T>
 __global__ void __launch_bounds__(kWideWarps * 32, kWideCtasPerSm)
 fuse_wide_kernel(int32_t C, int32_t stride, int32_t D, int32_t text_stride, int32_t split, const T *e_in,
-                 const T *e_text, FuseWorkspace ws, T *__restrict__ e_out, int32_t *__restrict__ pos,
-                 int32_t *__restrict__ len) {
+                 const T *e_text, FuseWorkspace ws, T *__restrict__ e_out, int32_t *__restrict__ pos) {
     constexpr int kElems = 16 / sizeof(T);
     ptx::grid_dependency_wait();
     const int b = blockIdx.y;
     const int32_t out_len = ws.seq_len[b];
-    if (blockIdx.x == 0 && threadIdx.x == 0) len[b] = out_len < 0 ? 0 : out_len;
     if (out_len < 0) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int vecs = D / kElems;
@@ -793,7 +800,7 @@ __global__ void __launch_bounds__(256) page_release_kernel(int64_t units, PageVi
 // Step 2: each unit takes the pages of slots [0, n] for its stage-1 length n (all or none; none
 // leaves page 0 missing, which the fusion and later calls read as "skipped").
 __global__ void __launch_bounds__(256) page_take_kernel(int64_t units, int32_t per_seq, FuseWorkspace ws, PageView pv,
-                                                        int32_t *status) {
+                                                        int32_t *len, int32_t *status) {
     ptx::grid_dependency_wait();
     const int64_t u = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
@@ -806,6 +813,7 @@ __global__ void __launch_bounds__(256) page_take_kernel(int64_t units, int32_t p
         if (top < need) {  // not enough: give them back (whatever other units did meanwhile)
             atomicAdd(pv.free_count, need);
             raise_status(status, VOXZIP_DEV_CAPACITY);
+            len[u] = 0;
             top = -1;
         }
     }
@@ -819,14 +827,15 @@ cudaError_t launch_slot_plan(int32_t B, int32_t capacity, int32_t stride, int32_
                              bool has_anchor, bool keep_bg, const int32_t *in_len, const int32_t *audio_begin,
                              const int32_t *audio_len, const int32_t *span_off, const int32_t *span_start,
                              const int32_t *span_end, const int32_t *span_groups, const FuseWorkspace &ws,
-                             int32_t *slot_map, int32_t *status, cudaStream_t stream) {
+                             int32_t *len, int32_t units_per_seq, int32_t *slot_map, int32_t *status,
+                             cudaStream_t stream) {
     cudaError_t err = launch_dependent(span_scan_kernel, dim3((unsigned)B), kScanThreads, 0, stream, B, stride, capacity,
                                        num_spans, anchor_stride, has_anchor, keep_bg, in_len, audio_begin, audio_len,
                                        span_off, span_start, span_end, span_groups, ws, status);
     if (err != cudaSuccess) return err;
     const dim3 grid_map((unsigned)((stride + kMapThreads - 1) / kMapThreads), (unsigned)B);
     return launch_dependent(slot_map_kernel, grid_map, kMapThreads, 0, stream, stride, keep_bg, in_len, audio_begin,
-                            audio_len, span_off, span_start, span_end, span_groups, ws, slot_map);
+                            audio_len, span_off, span_start, span_end, span_groups, ws, len, units_per_seq, slot_map);
 }
 
 }  // namespace
@@ -848,7 +857,8 @@ cudaError_t launch_anchor_fuse(const voxzip_cache_desc &d, const void *k_prefill
     ws.status = status;
     cudaError_t err = launch_slot_plan(d.batch, d.capacity, prefill_stride, num_spans, anchor_stride,
                                        anchor_k != nullptr, true, in_len, audio_begin, audio_len, span_off,
-                                       span_start, span_end, span_groups, ws, slot_map, status, stream);
+                                       span_start, span_end, span_groups, ws, len, d.layers * d.kv_heads, slot_map,
+                                       status, stream);
     if (err != cudaSuccess) return err;
     const bool bf16 = d.dtype == VOXZIP_BF16;
     if (d.head_dim == 128)
@@ -885,10 +895,11 @@ cudaError_t launch_anchor_fuse_paged(const voxzip_cache_desc &d, const voxzip_pa
     cudaError_t err = launch_dependent(page_release_kernel, dim3(blocks), 256, 0, stream, units, pv);
     if (err != cudaSuccess) return err;
     err = launch_slot_plan(d.batch, d.capacity, prefill_stride, num_spans, anchor_stride, anchor_k != nullptr, true,
-                           in_len, audio_begin, audio_len, span_off, span_start, span_end, span_groups, ws, slot_map,
-                           status, stream);
+                           in_len, audio_begin, audio_len, span_off, span_start, span_end, span_groups, ws, len,
+                           d.layers * d.kv_heads, slot_map, status, stream);
     if (err != cudaSuccess) return err;
-    err = launch_dependent(page_take_kernel, dim3(blocks), 256, 0, stream, units, d.layers * d.kv_heads, ws, pv, status);
+    err = launch_dependent(page_take_kernel, dim3(blocks), 256, 0, stream, units, d.layers * d.kv_heads, ws, pv, len,
+                           status);
     if (err != cudaSuccess) return err;
     const bool bf16 = d.dtype == VOXZIP_BF16;
     void *kc = pc.k_pool, *vc = pc.v_pool;
@@ -944,7 +955,7 @@ cudaError_t launch_embed_fuse(int32_t B, int32_t D, int32_t C, bool bf16, const 
     ws.status = status;
     cudaError_t err = launch_slot_plan(B, C, stride, num_spans, text_stride, e_text != nullptr, keep_background,
                                        in_len, audio_begin, audio_len, span_off, span_start, span_end, span_groups,
-                                       ws, slot_map, status, stream);
+                                       ws, len, 1, slot_map, status, stream);
     if (err != cudaSuccess) return err;
     // A grid-stride loop over (output row, column range) items on as many CTAs as are resident. Two
     // ranges from 96 vectors a row and four from 256: more items balance the warps better, until an item
@@ -957,9 +968,9 @@ cudaError_t launch_embed_fuse(int32_t B, int32_t D, int32_t C, bool bf16, const 
     using H = __nv_bfloat16;
     if (bf16)
         return launch_dependent(fuse_wide_kernel<H>, grid, kWideWarps * 32, 0, stream, C, stride, D, text_stride, split,
-                                (const H *)e_in, (const H *)e_text, ws, (H *)e_out, pos, len);
+                                (const H *)e_in, (const H *)e_text, ws, (H *)e_out, pos);
     return launch_dependent(fuse_wide_kernel<float>, grid, kWideWarps * 32, 0, stream, C, stride, D, text_stride, split,
-                            (const float *)e_in, (const float *)e_text, ws, (float *)e_out, pos, len);
+                            (const float *)e_in, (const float *)e_text, ws, (float *)e_out, pos);
 }
 
 }  // namespace voxzip

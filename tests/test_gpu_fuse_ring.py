@@ -1,6 +1,11 @@
 """Stage 1 at the edges of its ring kernels: spans shorter than, equal to and many times a ring stage,
 runs of output rows around a work item's, row widths around a team's columns, short, empty and skipped
-sequences beside long ones. Rows, positions, slot maps and lengths are the oracle's bit for bit."""
+sequences beside long ones. Rows, positions, slot maps and lengths are the oracle's bit for bit. A ring
+whose waits give up leaves every unit that it did not finish empty."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -134,3 +139,45 @@ def test_embedding_rows(dtype, width, text, keep):
         np.testing.assert_array_equal(out[b, :n].double().cpu().numpy(), r["stored"])
         np.testing.assert_array_equal(pos[b, :n].cpu().numpy(), r["pos"])
         assert not out[b, n:].any() and (pos[b, n:] == -7).all()
+
+
+GIVES_UP = """
+import sys
+import torch
+import paper_2608_08569_gb300._native as N
+N.LIB_PATH = sys.argv[1]
+from paper_2608_08569_gb300 import (DEV_TIMEOUT, CacheDesc, allocate_cache, allocate_paged_cache, voxzip_anchor_fuse,
+                                    voxzip_anchor_fuse_paged, voxzip_get_status)
+i32 = lambda x: torch.tensor(x, dtype=torch.int32, device="cuda")
+B, L, H, n, D = 2, 3, 2, 5000, 128
+ints = (i32([n, 40]), i32([0, 0]), i32([0, 0]), i32([0, 0, 0]), i32([]), i32([]), i32([]))
+for dtype in (torch.bfloat16, torch.float32):
+    desc = CacheDesc(B, L, 2 * H, H, D, 5056, dtype)
+    k = torch.ones(B, L, H, n, D, dtype=dtype, device="cuda")
+    c, p = allocate_cache(desc), allocate_paged_cache(desc, B * L * H * 80)
+    c["len"].fill_(7), p["len"].fill_(7)
+    voxzip_anchor_fuse(desc, k, k, *ints, c["k"], c["v"], c["score"], c["pos"], c["len"])
+    assert voxzip_get_status() == DEV_TIMEOUT
+    assert not c["len"].any(), c["len"]
+    voxzip_anchor_fuse_paged(desc, p, k, k, *ints)
+    assert voxzip_get_status() == DEV_TIMEOUT
+    assert not p["len"].any(), p["len"]
+"""
+
+
+@pytest.mark.skipif("VOXZIP_CHECKED" in os.environ, reason="builds a library of its own")
+def test_a_wait_that_gives_up_leaves_its_units_empty(tmp_path):
+    """A build whose waits for rows give up at once (the loads in flight are still waited for before a warp
+    leaves): the status word says so, and no unit keeps an earlier request's length."""
+    from paper_2608_08569_gb300 import build as B
+    objs = [os.path.join(B.BUILD_DIR, os.path.basename(s)[:-3] + ".o") for s in B._sources()]
+    if not all(os.path.exists(o) for o in objs):
+        B.build_library(force=True)
+    src, obj, lib = os.path.join(B.CSRC, "anchor_fuse.cu"), str(tmp_path / "anchor_fuse.o"), str(tmp_path / "lib.so")
+    cmds = [[B._nvcc(), *B.ARCH, *B.NVCC_FLAGS, "-DVOXZIP_FUSE_WAIT_LIMIT=0u", "-c", src, "-o", obj],
+            [B._nvcc(), *B.ARCH, "-shared", "-cudart", "shared", "-Xlinker", "-rpath,/usr/local/cuda/lib64", "-o", lib, obj,
+             *[o for o in objs if os.path.basename(o) != "anchor_fuse.o"]],
+            [sys.executable, "-c", GIVES_UP, lib]]
+    for cmd in cmds:
+        r = subprocess.run(cmd, cwd=B.ROOT, capture_output=True, text=True, timeout=600)
+        assert r.returncode == 0, r.stderr[-3000:]

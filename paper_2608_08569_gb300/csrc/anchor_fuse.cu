@@ -680,13 +680,19 @@ cudaError_t launch_fuse_rows(const voxzip_cache_desc &d, int32_t stride, int32_t
     // CTAs on half the SMs already keep the link busy (on GB300: 87 ms for the 18.1 GB of a 60-min
     // request, ~209 GB/s), and the rest of the GPU stays free for a kernel running beside it: a decode
     // loop of another request slows by ~2% (by 67% when every SM also runs a stage-1 CTA).
-    cudaPointerAttributes pa{};
-    const bool host_rows = cudaPointerGetAttributes(&pa, kp) == cudaSuccess && pa.type == cudaMemoryTypeHost;
-    cudaGetLastError();
-    // Rows of 128 bytes (bf16, D = 64) would leave half of the ring kernel's lanes idle, and rows in host
-    // memory are bound by the link: both keep fuse_rows_kernel.
+    auto memory = [](const void *p) {
+        cudaPointerAttributes pa{};
+        if (cudaPointerGetAttributes(&pa, p) == cudaSuccess) return pa.type;
+        cudaGetLastError();
+        return cudaMemoryTypeUnregistered;
+    };
+    const cudaMemoryType mk = memory(kp), mv = memory(vp);
+    const bool host_rows = mk == cudaMemoryTypeHost || mv == cudaMemoryTypeHost;
+    // Rows of 128 bytes (bf16, D = 64) would leave half of the ring kernel's lanes idle, and rows that are
+    // not both in device memory are bound by the link: both keep fuse_rows_kernel, whose plain loads any
+    // memory serves.
     using FR = FuseRing<T, D>;
-    if constexpr (FR::kRowBytes >= 256) if (!host_rows) {
+    if constexpr (FR::kRowBytes >= 256) if (mk == cudaMemoryTypeDevice && mv == cudaMemoryTypeDevice) {
         static std::atomic<uint64_t> configured{0};
         const cudaError_t set = once_per_device(configured, [] {
             return cudaFuncSetAttribute(fuse_ring_kernel<T, D, kPaged>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -141,6 +141,39 @@ def test_embedding_rows(dtype, width, text, keep):
         assert not out[b, n:].any() and (pos[b, n:] == -7).all()
 
 
+@pytest.mark.parametrize("paged", [False, True])
+@pytest.mark.parametrize("host", ["k", "v"])
+def test_only_one_of_the_two_prefills_in_host_memory(paged, host):
+    """K in pinned host memory and V on the device, or the other way round: the same rows."""
+    seqs, ints, stride, _ = _batch(np.random.default_rng(17))
+    B, L, H, D, C = len(seqs), 1, 2, 128, (stride + 63) // 64 * 64
+    desc = CacheDesc(B, L, 2 * H, H, D, C, torch.bfloat16)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    dev = [torch.randn(B, L, H, stride, D, generator=g, device="cuda").bfloat16() for _ in range(2)]
+    mixed = [x.cpu().pin_memory() if y == host else x for x, y in zip(dev, "kv")]
+    got = []
+    for k, v in (dev, mixed):
+        if paged:
+            c = allocate_paged_cache(desc, B * L * H * (C // 64 + 1))
+            voxzip_anchor_fuse_paged(desc, c, k, v, *ints, workspace=torch.empty(1 << 22, dtype=torch.uint8, device="cuda"))
+            table = c["page_table"].long().clamp(min=0)
+            rows = [c[x][table].reshape(B, L, H, C, D) for x in ("k_pool", "v_pool")]
+        else:
+            c = allocate_cache(desc)
+            voxzip_anchor_fuse(desc, k, v, *ints, c["k"], c["v"], c["score"], c["pos"], c["len"])
+            rows = [c["k"], c["v"]]
+        assert voxzip_get_status() == DEV_BAD_SPANS
+        got.append((c["len"], c["pos"], rows))
+    (la, pa, ra), (lb, pb, rb) = got
+    assert torch.equal(la, lb) and la.any()
+    for b in range(B):
+        n = int(la[b, 0, 0])
+        assert torch.equal(pa[b, ..., :n], pb[b, ..., :n])
+        for x, y in zip(ra, rb):
+            assert torch.equal(x[b, :, :, :n], y[b, :, :, :n])
+
+
 GIVES_UP = """
 import sys
 import torch

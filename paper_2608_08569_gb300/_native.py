@@ -7,6 +7,7 @@ library's CUDA kernels; there is no fallback when the library is missing.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 import threading
 from dataclasses import dataclass
@@ -56,25 +57,32 @@ class CacheDesc:
     def group(self) -> int:
         return self.q_heads // self.kv_heads
 
-    def __post_init__(self):
-        # What every call needs of the (immutable) descriptor, made once.
-        put, units = object.__setattr__, (self.batch, self.layers, self.kv_heads)
-        put(self, "_units", units)
-        put(self, "_slots", units + (self.capacity,))
-        put(self, "_rows", units + (self.capacity, self.head_dim))
-        try:
-            put(self, "_c", self.c_struct())
-        except (KeyError, TypeError):  # raised again by the call that uses the descriptor
-            put(self, "_c", None)
+    # What every call needs of the (immutable) descriptor, made at its first use: a descriptor that was
+    # pickled by an earlier version, or whose class has a __post_init__ of its own, has it too.
+    @functools.cached_property
+    def _units(self):
+        return self.batch, self.layers, self.kv_heads
+
+    @functools.cached_property
+    def _slots(self):
+        return self._units + (self.capacity,)
+
+    @functools.cached_property
+    def _rows(self):
+        return self._slots + (self.head_dim,)
+
+    @functools.cached_property
+    def _c(self):
+        """The binding's own C struct (never handed out: c_struct makes a new one)."""
+        return self.c_struct()
+
+    def __getstate__(self):  # pickles and copies hold the fields alone
+        return {k: v for k, v in self.__dict__.items()
+                if not isinstance(getattr(type(self), k, None), functools.cached_property)}
 
     def c_struct(self) -> _Desc:
         return _Desc(self.batch, self.layers, self.q_heads, self.kv_heads, self.head_dim, self.capacity,
                      _DTYPES[self.dtype])
-
-
-def _c_desc(desc: CacheDesc) -> _Desc:
-    """The binding's own C struct of a descriptor (never handed out: c_struct makes a new one)."""
-    return desc._c if desc._c is not None else desc.c_struct()
 
 
 class _EmbedDesc(ctypes.Structure):
@@ -269,7 +277,7 @@ def _check_dense_state(desc: CacheDesc, score, pos, len_) -> None:
 
 def voxzip_paged_init(desc: CacheDesc, pc, stream=None) -> None:
     """Empties every unit of a paged cache (page u for unit u's slot 0, the rest free)."""
-    d, ps = _c_desc(desc), _paged_struct(desc, pc)
+    d, ps = desc._c, _paged_struct(desc, pc)
     _need(pc["len"], "len", torch.int32, (desc.batch, desc.layers, desc.kv_heads))
     _check("voxzip_paged_init", lib().voxzip_paged_init(ctypes.byref(d), ctypes.byref(ps), _ptr(pc["len"]),
                                                         _stream(stream)))
@@ -303,7 +311,7 @@ def voxzip_anchor_fuse_paged(desc: CacheDesc, pc, k_prefill, v_prefill, in_len, 
         anchor_stride = anchor_k.shape[3]
         _need(anchor_k, "anchor_k", desc.dtype, (B, L, H, anchor_stride, D))
         _need(anchor_v, "anchor_v", desc.dtype, (B, L, H, anchor_stride, D))
-    d, ps = _c_desc(desc), _paged_struct(desc, pc)
+    d, ps = desc._c, _paged_struct(desc, pc)
     need = int(lib().voxzip_anchor_fuse_paged_workspace_size(ctypes.byref(d), int(stride), int(num_spans)))
     if workspace is None or workspace.numel() < need:
         workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=k_prefill.device)
@@ -325,7 +333,7 @@ def voxzip_decode_step_paged(desc: CacheDesc, pc, layer_begin: int, layer_count:
     _need(out, "out", desc.dtype, (layer_count, B, Hq, D))
     _need(new_pos, "new_pos", torch.int32, (B,))
     _check_dense_state(desc, pc["score"], pc["pos"], pc["len"])
-    d, ps = _c_desc(desc), _paged_struct(desc, pc)
+    d, ps = desc._c, _paged_struct(desc, pc)
     _check("voxzip_decode_step_paged", lib().voxzip_decode_step_paged(
         ctypes.byref(d), ctypes.byref(ps), int(layer_begin), int(layer_count), _ptr(q), _ptr(k_new), _ptr(v_new),
         _ptr(new_pos), _ptr(pc["score"]), _ptr(pc["pos"]), _ptr(pc["len"]), float(gamma), float(sm_scale),
@@ -348,14 +356,14 @@ def voxzip_evict_paged(desc: CacheDesc, pc, layer_begin: int, layer_count: int, 
         raise ValueError("compaction must be 'ordered' or 'fill'")
     pol = _EvictPolicy(int(sink), float(recent_frac), int(bool(history)), sb, sl,
                        VOXZIP_COMPACT_FILL if compaction == "fill" else VOXZIP_COMPACT_ORDERED)
-    d, ps = _c_desc(desc), _paged_struct(desc, pc)
+    d, ps = desc._c, _paged_struct(desc, pc)
     _check("voxzip_evict_paged", lib().voxzip_evict_paged(
         ctypes.byref(d), ctypes.byref(ps), int(layer_begin), int(layer_count), _ptr(pc["score"]), _ptr(pc["pos"]),
         _ptr(pc["len"]), _ptr(budget), ctypes.byref(pol), _stream(stream)))
 
 
 def voxzip_anchor_fuse_workspace_size(desc: CacheDesc, prefill_stride: int, num_spans: int) -> int:
-    d = _c_desc(desc)
+    d = desc._c
     return int(lib().voxzip_anchor_fuse_workspace_size(ctypes.byref(d), int(prefill_stride), int(num_spans)))
 
 
@@ -387,7 +395,7 @@ def voxzip_anchor_fuse(desc: CacheDesc, k_prefill, v_prefill, in_len, audio_begi
     if workspace is None:
         workspace = torch.empty(max(need, 256), dtype=torch.uint8, device=k_cache.device)
     _need(workspace, "workspace", torch.uint8)
-    d = _c_desc(desc)
+    d = desc._c
     _check("voxzip_anchor_fuse", lib().voxzip_anchor_fuse(
         ctypes.byref(d), _ptr(k_prefill), _ptr(v_prefill), int(stride), _ptr(in_len), _ptr(audio_begin),
         _ptr(audio_len), _ptr(span_off), int(num_spans), _ptr(span_start), _ptr(span_end), _ptr(span_groups),
@@ -485,7 +493,7 @@ def voxzip_anchor_fuse_noalloc(desc: CacheDesc, k_prefill, v_prefill, in_len, au
         anchor_stride = anchor_k.shape[3]
         _need(anchor_k, "anchor_k", desc.dtype, (B, L, H, anchor_stride, D))
         _need(anchor_v, "anchor_v", desc.dtype, (B, L, H, anchor_stride, D))
-    d = _c_desc(desc)
+    d = desc._c
     _check("voxzip_anchor_fuse_noalloc", lib().voxzip_anchor_fuse_noalloc(
         ctypes.byref(d), _ptr(k_prefill), _ptr(v_prefill), int(stride), _ptr(in_len), _ptr(audio_begin),
         _ptr(audio_len), _ptr(span_off), int(num_spans), _ptr(span_start), _ptr(span_end), _ptr(span_groups),
@@ -504,7 +512,7 @@ def voxzip_decode_step(desc: CacheDesc, layer_begin: int, layer_count: int, q, k
     _need(out, "out", desc.dtype, (layer_count, B, Hq, D))
     _need(new_pos, "new_pos", torch.int32, (B,))
     _check_cache(desc, k_cache, v_cache, score, pos, len_)
-    d = _c_desc(desc)
+    d = desc._c
     _check("voxzip_decode_step", lib().voxzip_decode_step(
         ctypes.byref(d), int(layer_begin), int(layer_count), _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(new_pos),
         _ptr(k_cache), _ptr(v_cache), _ptr(score), _ptr(pos), _ptr(len_), float(gamma), float(sm_scale),
@@ -516,7 +524,7 @@ def voxzip_evict(desc: CacheDesc, layer_begin: int, layer_count: int, k_cache, v
     """Budgeted eviction (Eq. 7-9) for layers [layer_begin, layer_begin + layer_count)."""
     _check_cache(desc, k_cache, v_cache, score, pos, len_)
     _need(budget, "budget", torch.int32, (desc.batch,))
-    d = _c_desc(desc)
+    d = desc._c
     _check("voxzip_evict", lib().voxzip_evict(
         ctypes.byref(d), int(layer_begin), int(layer_count), _ptr(k_cache), _ptr(v_cache), _ptr(score), _ptr(pos),
         _ptr(len_), _ptr(budget), int(sink), float(recent_frac), _stream(stream)))
@@ -540,7 +548,7 @@ def voxzip_evict_ex(desc: CacheDesc, layer_begin: int, layer_count: int, k_cache
         raise ValueError("compaction must be 'ordered' or 'fill'")
     pol = _EvictPolicy(int(sink), float(recent_frac), int(bool(history)), sb, sl,
                        VOXZIP_COMPACT_FILL if compaction == "fill" else VOXZIP_COMPACT_ORDERED)
-    d = _c_desc(desc)
+    d = desc._c
     _check("voxzip_evict_ex", lib().voxzip_evict_ex(
         ctypes.byref(d), int(layer_begin), int(layer_count), _ptr(k_cache), _ptr(v_cache), _ptr(score), _ptr(pos),
         _ptr(len_), _ptr(budget), ctypes.byref(pol), _stream(stream)))

@@ -207,3 +207,35 @@ def test_prefill_may_be_pinned_host_memory_other_tensors_not():
             N._need(torch.zeros(4, dtype=torch.bfloat16), "k_prefill", torch.bfloat16, pinned_ok=True)
     with pytest.raises(ValueError, match="on a CUDA device"):
         N._need(torch.zeros(4, dtype=torch.int32), "in_len", torch.int32)
+
+
+def test_descriptors_from_older_pickles_and_subclasses_work():
+    """A call needs nothing of a CacheDesc but its fields: one restored from a pickle that holds only
+    those, or of a subclass with a __post_init__ of its own, sizes and checks calls like any other; a
+    used one still pickles and copies as its fields; a dtype without a C value is refused by the call."""
+    import copy
+    import dataclasses
+    import pickle
+    import paper_2608_08569_gb300 as V
+
+    @dataclasses.dataclass(frozen=True)
+    class Named(V.CacheDesc):
+        name: str = "x"
+
+        def __post_init__(self):
+            assert self.layers > 0
+
+    made = V.CacheDesc(2, 3, 8, 2, 64, 128, torch.float32)
+    old = object.__new__(V.CacheDesc)
+    old.__dict__.update(dataclasses.asdict(made))
+    want = V.voxzip_anchor_fuse_workspace_size(made, 100, 4)
+    assert want > 0
+    for d in (old, Named(2, 3, 8, 2, 64, 128, torch.float32), pickle.loads(pickle.dumps(made)), copy.deepcopy(made),
+              dataclasses.replace(made)):
+        assert V.voxzip_anchor_fuse_workspace_size(d, 100, 4) == want
+        with pytest.raises(ValueError, match="k_cache"):
+            V.voxzip_evict(d, 0, 1, *[torch.zeros(1)] * 6)
+    assert old == made and hash(old) == hash(made)
+    assert set(pickle.loads(pickle.dumps(made)).__dict__) == {f.name for f in dataclasses.fields(made)}
+    with pytest.raises(KeyError):
+        V.voxzip_anchor_fuse_workspace_size(V.CacheDesc(2, 3, 8, 2, 64, 128, torch.float16), 100, 4)

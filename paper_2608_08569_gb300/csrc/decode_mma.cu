@@ -193,15 +193,16 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
     // for that atomically, past L1: it may be about to change, so it only aims the prefetch.
     // Back-to-back launches, against K rows only and the host's length bound: 32 ragged sequences, one
     // layer each, 21.1 -> 20.2 us; 16 units of 6 400 rows 14.4 -> 13.3; more rows than that gain nothing.
-    int est_j0 = 0, est_cnt = 0;
+    int est_j0 = 0, est_cnt = 0, seen = 0;
+    if (warp == kConsumerWarps) seen = ptx::load_relaxed(p.len + ui.cache_unit);
+    __syncthreads();  // the ring is set up (the length is still on its way: no other warp waits for it)
     if (warp == kConsumerWarps) {
-        const int seen = min(max(ptx::load_relaxed(p.len + ui.cache_unit), 0), p.C - 1) + 1;
+        seen = min(max(seen, 0), p.C - 1) + 1;
         const int est_chunk = range_of<kPaged>(seen, S);
         est_j0 = min(seen, rank * est_chunk);
         est_cnt = min(seen, est_j0 + est_chunk) - est_j0;
         prefetch_rows<D, kPaged>(p, ui.cache_unit, est_j0, est_cnt, kAheadRows);
     }
-    __syncthreads();
     // Everything from here on reads what the previous kernel wrote (lengths, pages, cache rows,
     // scores, queries): wait for its completion.
     ptx::grid_dependency_wait();

@@ -50,3 +50,18 @@ def test_decode_plans_are_kept_per_device():
 def test_another_units_length_is_read_atomically():
     """The cluster of a later unit may run beside this one and store that unit's length."""
     assert not re.findall(r"p\.len\[(?!ui\.cache_unit\])", SOURCES["decode_mma.cu"])
+
+
+def test_the_logits_of_a_lane_group_lie_in_different_banks():
+    """Phase V of the decode reads, per lane (g, qd), head 8 nt + g of row qd + 4 e: with the row length and
+    the swap of its template, no two lanes of a warp meet in a bank. The swapped column is a permutation."""
+    s = SOURCES["decode_mma.cu"]
+    assert "return kSwap ? h ^ ((row & 2) << 2) : h;" in s and "kSwap = NT == 2 && (kCluster || D == 64)" in s
+    for heads, swap in ((8, False), (16, True)):
+        col = lambda row, h: h ^ ((row & 2) << 2) if swap else h
+        for row in range(16):
+            assert sorted(col(row, h) for h in range(heads)) == list(range(heads))
+        for nt in range(heads // 8):
+            for e in range(4):
+                at = [(qd + 4 * e) * heads + col(qd + 4 * e, nt * 8 + g) for g in range(8) for qd in range(4)]
+                assert len({a % 32 for a in at}) == 32

@@ -881,11 +881,14 @@ struct Plan {
     int clusters;  // resident at once
 };
 
-// Constants of the planner's time model, fitted to 1 985 timings of forced plans on GB300 (D = 128):
-// launches of 4 to 1 536 units of 60 to 11 520 rows, one layer or all, every S and NS, back to back in a
-// CUDA graph. The plans it picks are 0.7% slower on average than the best of each shape (11% at worst)
-// where the rows come from HBM, and 0.3% (6%) where they stay in L2; the constants that went before
-// (5 us fixed, 20 rows/us a stage, 90 an SM, no cost of sharing an SM) took 4.2% (53%) on the first.
+// Constants of the planner's time model, fitted to timings of forced plans on GB300, back to back in a CUDA
+// graph: launches of 1 to 4 416 units of 34 to 12 000 rows, one layer or all, every S and NS, groups of 2, 8
+// and 16 heads; D = 128 and D = 64 each where the rows come from HBM and where they stay in L2. Over those
+// shapes the plans it picks are slower than the best of each by, on average and at worst:
+//   D = 128  HBM 1.5%, 10% (141 shapes)    L2 2.6%, 18% (127)
+//   D = 64   HBM 0.5%, 14% (107)           L2 1.8%, 23% (147)
+// With the constants of D = 128 (and 128 / D as many rows per SM) D = 64 took 2.9%, 26% and 3.3%, 30%; without
+// full_us a launch of 36 units of 4 100 rows took rings of four stages, 17.1 us, where three take 14.3.
 struct PlanModel {
     double fixed_us;           // a CTA's prologue and epilogue
     double shared_us;          // more for each CTA that shares its SM
@@ -896,10 +899,14 @@ struct PlanModel {
     double sm_rows_per_us;     // what the CTAs of an SM share
     double last_round;         // how far a part-filled last round costs a whole one
     double next_us;            // what a round of clusters saves when the one before asks L2 for its first rows
+    double full_us;            // a launch that takes all the room leaves none for the next one's CTAs to start in
 };
-constexpr PlanModel kPlanHbm{4.3, 0.88, 0.2, 0.6, 25.9, 81.0, 163.0, 0.77, 1.2};
+constexpr PlanModel kPlanHbm128{4.3, 0.88, 0.2, 0.6, 25.9, 81.0, 163.0, 0.77, 1.2, 1.0};
+constexpr PlanModel kPlanHbm64{4.6, 0.8, 1.4, 2.0, 28.8, 66.0, 334.0, 0.95, 0.7, 1.5};
 // A cache that fits comfortably in L2 as a whole: in a decode loop it stays there from step to step.
-constexpr PlanModel kPlanL2{5.0, 0.69, 0.2, 1.4, 28.4, 85.0, 221.0, 0.36, 0.0};  // three stages keep the warps fed
+constexpr PlanModel kPlanL2x128{5.0, 0.69, 0.2, 1.4, 28.4, 85.0, 221.0, 0.36, 0.0, 0.0};  // three stages keep the warps fed
+constexpr PlanModel kPlanL2x64{5.0, 0.7, 0.1, 0.7, 34.0, 111.0, 441.0, 0.39, 0.0, 0.0};
+constexpr double kFullFrom = 0.9;  // share of the resident clusters from which full_us counts
 constexpr double kL2ResidentBytes = 64.0 * 1048576.0;
 
 // Chooses the cluster size S and ring depth NS with a time model. For each (S, NS) the CTAs hold
@@ -909,7 +916,7 @@ constexpr double kL2ResidentBytes = 64.0 * 1048576.0;
 // plus its tokens at one CTA's streaming rate, which grows with the ring stages in flight until its
 // consumer warps or the CTAs that share its SM bound it.
 Plan plan(int D, int NT, int units, int nmax, bool paged, bool l2) {
-    const PlanModel &md = l2 ? kPlanL2 : kPlanHbm;
+    const PlanModel &md = l2 ? (D == 64 ? kPlanL2x64 : kPlanL2x128) : (D == 64 ? kPlanHbm64 : kPlanHbm128);
     const int nmid = max(1, nmax - kTile / 2);  // nmax is a bucket's upper end
     Plan best{0, 3, 0, 0};
     double best_cost = 0.0;
@@ -931,14 +938,14 @@ Plan plan(int D, int NT, int units, int nmax, bool paged, bool l2) {
             const int cl = dispatch(D, NT, ns, [&](auto k) { return max_active_clusters<decltype(k)>(S, sm); });
             if (cl <= 0) continue;
             const double per_sm = fmax(1.0, (double)min(units, cl) * S / sms);  // CTAs sharing an SM
-            const double rate = fmin(fmin(md.stage_rows_per_us * ns, md.cta_rows_per_us),
-                                     md.sm_rows_per_us * (128.0 / D) / per_sm);  // shorter rows: more of them
+            const double rate = fmin(fmin(md.stage_rows_per_us * ns, md.cta_rows_per_us), md.sm_rows_per_us / per_sm);
             const double fixed = md.fixed_us + md.shared_us * (per_sm - 1.0) + (S > 1 ? md.cluster_us : 0.0) +
                                  (S == 16 ? md.cluster16_us : 0.0);
             const double share = (double)units / cl;
             const double rounds = share <= 1.0 ? 1.0 : md.last_round * ceil(share) + (1.0 - md.last_round) * share;
+            const double full = share <= 1.0 ? fmax(0.0, share - kFullFrom) / (1.0 - kFullFrom) * md.full_us : 0.0;
             const double cost = rounds * (fixed + (double)((nmid + S - 1) / S) / rate) -
-                                (S > 1 ? (rounds - 1.0) * md.next_us : 0.0);
+                                (S > 1 ? (rounds - 1.0) * md.next_us : 0.0) + full;
             if (best.S == 0 || cost < best_cost) {
                 best = Plan{S, ns, cap, cl};
                 best_cost = cost;

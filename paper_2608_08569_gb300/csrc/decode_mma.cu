@@ -201,10 +201,13 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
     // for that atomically, past L1: it may be about to change, so it only aims the prefetch.
     // Back-to-back launches, against K rows only and the host's length bound: 32 ragged sequences, one
     // layer each, 21.1 -> 20.2 us; 16 units of 6 400 rows 14.4 -> 13.3; more rows than that gain nothing.
+    // A consumer warp does it, since its first tile comes a memory latency after the producer's length; when
+    // paged the producer, which needs the predicted range.
+    constexpr int kAimWarp = kPaged ? kConsumerWarps : kConsumerWarps - 1;
     int est_j0 = 0, est_cnt = 0, seen = 0;
-    if (warp == kConsumerWarps) seen = ptx::load_relaxed(p.len + ui.cache_unit);
+    if (warp == kAimWarp) seen = ptx::load_relaxed(p.len + ui.cache_unit);
     __syncthreads();  // the ring is set up (the length is still on its way: no other warp waits for it)
-    if (warp == kConsumerWarps) {
+    if (warp == kAimWarp) {
         seen = min(max(seen, 0), p.C - 1) + 1;
         const int est_chunk = range_of<kPaged>(seen, S);
         est_j0 = min(seen, rank * est_chunk);

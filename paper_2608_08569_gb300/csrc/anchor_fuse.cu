@@ -137,9 +137,9 @@ __host__ __device__ inline size_t carve(const voxzip_cache_desc &d, int32_t stri
     return off;
 }
 
-// Launches a kernel of the stage as a programmatic dependent of the kernel before it on the stream: its
-// CTAs start while that one drains, and wait for it (griddepcontrol.wait) before their first access.
-// The gaps between the three launches took 6 us of every call: embeddings of 4 x 60 min 223.3 -> 217.6 us,
+// Launches a kernel of the stage as a programmatic dependent of the kernel before it on the stream: it is
+// launched as the last CTAs of that one exit (no kernel of the stage lets it start earlier), and waits for its
+// writes (griddepcontrol.wait) before its first access. What it saves is launch latency: the gaps between the three launches took 6 us of every call: embeddings of 4 x 60 min 223.3 -> 217.6 us,
 // of 10 min 24.0 -> 20.2; K/V of 10 min, 192 units, 180 -> 174, of a 30-s clip 38.2 -> 31.9.
 // The first kernel may be resident while the caller's last one still writes its inputs, so no kernel takes
 // them as `const __restrict__`, which would allow read-only loads (four 60-min prompts 3 843 us with, 3 844 without).
@@ -448,13 +448,6 @@ constexpr uint32_t kFuseWaitLimit = 1u << 22;  // polls before an mbarrier wait 
 #define VOXZIP_FUSE_WAIT_LIMIT kFuseWaitLimit  // of a wait for rows (0 in a test's build: every wait gives up)
 #endif
 
-__device__ __forceinline__ void bulk_load(void *smem_dst, const void *src, uint32_t bytes, uint64_t *bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     ptx::smem_u32(smem_dst)),
-                 "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(ptx::smem_u32(bar))
-                 : "memory");
-}
-
 template <typename T, int D, bool kPaged>
 __global__ void __launch_bounds__(FuseRing<T, D>::kWarps * 32, 1)
 fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, int32_t anchor_stride,
@@ -464,7 +457,8 @@ fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
     using FR = FuseRing<T, D>;
     constexpr int kElems = 16 / (int)sizeof(T);
     constexpr int kRowVecs = D / kElems;                              // 16-byte vectors of a row
-    constexpr int kPer = 2 * kRowVecs > 32 ? 2 * kRowVecs / 32 : 1;  // vectors per lane: of K, then of V
+    static_assert(FR::kRowBytes >= 256, "every lane owns a vector");
+    constexpr int kPer = 2 * kRowVecs / 32;  // vectors per lane: of K, then of V
     constexpr int kR = FR::kRows, kDepth = FR::kDepth;
     extern __shared__ __align__(128) uint8_t ring_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -545,8 +539,8 @@ fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
                 uint64_t *bar = &full[filled % kDepth];
                 const int64_t src = ((int64_t)p_u * stride + p_row) * D;
                 ptx::mbar_arrive_expect_tx(bar, 2u * (uint32_t)rows * FR::kRowBytes);
-                bulk_load(dst, k_prefill + src, (uint32_t)rows * FR::kRowBytes, bar);
-                bulk_load(dst + kR * FR::kRowBytes, v_prefill + src, (uint32_t)rows * FR::kRowBytes, bar);
+                ptx::bulk_load(dst, k_prefill + src, (uint32_t)rows * FR::kRowBytes, bar);
+                ptx::bulk_load(dst + kR * FR::kRowBytes, v_prefill + src, (uint32_t)rows * FR::kRowBytes, bar);
             }
             p_row += rows;
             ++filled;
@@ -554,8 +548,7 @@ fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
     };
     refill();
 
-    // This lane's vectors: of the K row for v < kRowVecs, of the V row after.
-    const bool active = lane < 2 * kRowVecs;
+    // A lane's vectors v: of the K row for v < kRowVecs, of the V row after.
     bool ok = true;
     while (cur.n > 0 && ok) {
         if (lane < cur.n) {
@@ -573,7 +566,7 @@ fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
             const int32_t o_row = kPaged ? __shfl_sync(0xffffffffu, cur.o, k) : cur.slot0 + k;
             const bool anchored = a_row >= 0 && VOXZIP_IN_RANGE(ws.status, a_row < anchor_stride);
             uint4 anc[kPer];
-            if (anchored && active) {
+            if (anchored) {
 #pragma unroll
                 for (int i = 0; i < kPer; ++i) {
                     const int v = lane + 32 * i;
@@ -608,9 +601,8 @@ fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
 #pragma unroll
                     for (int i = 0; i < kPer; ++i) {
                         const int v = lane + 32 * i;
-                        if (active)
-                            accumulate16<T>(acc[i], *reinterpret_cast<const uint4 *>(
-                                                        at + (v < kRowVecs ? 0 : kR * FR::kRowBytes) + v % kRowVecs * 16));
+                        accumulate16<T>(acc[i], *reinterpret_cast<const uint4 *>(
+                                                    at + (v < kRowVecs ? 0 : kR * FR::kRowBytes) + v % kRowVecs * 16));
                     }
                     at += FR::kRowBytes;
                 }
@@ -618,26 +610,24 @@ fuse_ring_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
                 r += take;
             }
             if (!ok) break;
-            if (active) {
-                T *out[2] = {k_cache + out_base + (int64_t)o_row * D, v_cache + out_base + (int64_t)o_row * D};
+            T *out[2] = {k_cache + out_base + (int64_t)o_row * D, v_cache + out_base + (int64_t)o_row * D};
 #pragma unroll
-                for (int i = 0; i < kPer; ++i) {
-                    const int v = lane + 32 * i;
-                    if (r1 - r0 > 1) {
-                        const float cnt = (float)(r1 - r0);
+            for (int i = 0; i < kPer; ++i) {
+                const int v = lane + 32 * i;
+                if (r1 - r0 > 1) {
+                    const float cnt = (float)(r1 - r0);
 #pragma unroll
-                        for (int e = 0; e < kElems; ++e) acc[i][e] = __fdiv_rn(acc[i][e], cnt);
-                    }
-                    if (anchored) {
-                        float t[kElems];
-#pragma unroll
-                        for (int e = 0; e < kElems; ++e) t[e] = 0.f;
-                        accumulate16<T>(t, anc[i]);
-#pragma unroll
-                        for (int e = 0; e < kElems; ++e) acc[i][e] = __fadd_rn(acc[i][e], t[e]);
-                    }
-                    *reinterpret_cast<uint4 *>((v < kRowVecs ? out[0] : out[1]) + v % kRowVecs * kElems) = pack16<T>(acc[i]);
+                    for (int e = 0; e < kElems; ++e) acc[i][e] = __fdiv_rn(acc[i][e], cnt);
                 }
+                if (anchored) {
+                    float t[kElems];
+#pragma unroll
+                    for (int e = 0; e < kElems; ++e) t[e] = 0.f;
+                    accumulate16<T>(t, anc[i]);
+#pragma unroll
+                    for (int e = 0; e < kElems; ++e) acc[i][e] = __fadd_rn(acc[i][e], t[e]);
+                }
+                *reinterpret_cast<uint4 *>((v < kRowVecs ? out[0] : out[1]) + v % kRowVecs * kElems) = pack16<T>(acc[i]);
             }
         }
         if (!ok) break;

@@ -35,15 +35,6 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16 *p) {
     r.w = __uint_as_float(u.y & 0xffff0000u);
     return r;
 }
-__device__ __forceinline__ void store4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
-__device__ __forceinline__ void store4(__nv_bfloat16 *p, float4 v) {
-    __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y);
-    __nv_bfloat162 b = __floats2bfloat162_rn(v.z, v.w);
-    uint2 u;
-    u.x = *reinterpret_cast<uint32_t *>(&a);
-    u.y = *reinterpret_cast<uint32_t *>(&b);
-    *reinterpret_cast<uint2 *>(p) = u;
-}
 
 __device__ __forceinline__ void raise_status(int32_t *status, uint32_t bits) {
     atomicOr(reinterpret_cast<unsigned int *>(status), bits);

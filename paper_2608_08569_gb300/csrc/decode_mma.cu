@@ -143,9 +143,10 @@ __device__ __forceinline__ void prefetch_rows(const MmaParams &p, int64_t cache_
 // kCluster: launched in clusters of S > 1 CTAs (else one CTA holds the whole unit).
 // kPaged: K/V rows live in page pools (see paged.cuh).
 // kNext: the launch has more clusters than are resident at once, so a CTA's place is taken by a later
-// one; its first rows are requested into L2 while this one finishes (60-min 20x, 768 units: 156 -> 152 us a
-// step, and 148 with the 4-CTA clusters in seven rounds that then pay). An instantiation of its own: in launches of one round, the test alone
-// cost 1-2%. Without a cluster the CTAs of an SM are not in step, and it gained nothing.
+// one; its first rows are requested into L2 while this one finishes. A step of 60-min 20x (768 units) went
+// from 156 to 152 us with it, and to 148 with clusters of 4 CTAs in seven rounds, which pay only then. An
+// instantiation of its own: in launches of one round, the test alone cost 1-2%. Without a cluster the CTAs of
+// an SM are not in step, and it gained nothing.
 template <int D, int NT, int kStages, bool kCluster, bool kPaged, bool kNext>
 __global__ void __launch_bounds__(kThreads)
 decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant__ CUtensorMap tmv,
@@ -195,7 +196,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
         ptx::fence_mbar_init();
     }
     // Launched as a programmatic dependent of the previous kernel on the stream, the CTA may start
-    // before that kernel ends. Until then nothing that it writes may be read, but L2 can be asked for
+    // before that kernel ends. Until then nothing that it writes may be used, but L2 can be asked for
     // this CTA's first rows while the previous launch drains and HBM idles: K rows, then V rows where
     // the K range is short, as many as fill the ring (three tiles at least). The unit's length is read
     // for that atomically, past L1: it may be about to change, so it only aims the prefetch.
@@ -277,7 +278,7 @@ decode_mma_kernel(const __grid_constant__ CUtensorMap tmk, const __grid_constant
     // warp that owns that row of its tile loads k_new / v_new into registers here, writes them over
     // the row the TMA brought in, so no load waits for the store, and stores them (with the position)
     // to the cache for later steps when it patches that tile: a store issued here would wait for its
-    // load and hold back the barrier before the ring's first load.
+    // load, and the warp's first tile behind it.
     const int jn = n - 1 - j0;
     const bool own_new = jn >= 0 && jn < cnt;
     const int t_new = own_new ? jn / kTile : -1;

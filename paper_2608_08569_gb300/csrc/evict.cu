@@ -72,14 +72,8 @@ struct BulkRing {
     static_assert(kDepth >= 3, "a sub-chunk in flight and two stores draining");
 };
 
-// 1-D bulk copies (the async proxy): global -> shared counted on an mbarrier, shared -> global in
-// bulk groups. Addresses 16-byte aligned, sizes multiples of 16.
-__device__ __forceinline__ void bulk_load(void *smem_dst, const void *src, uint32_t bytes, uint64_t *bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     ptx::smem_u32(smem_dst)),
-                 "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(ptx::smem_u32(bar))
-                 : "memory");
-}
+// 1-D bulk copies (the async proxy) from shared to global memory, in bulk groups. Addresses 16-byte aligned,
+// sizes multiples of 16.
 __device__ __forceinline__ void bulk_store(void *dst, const void *smem_src, uint32_t bytes) {
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(reinterpret_cast<uint64_t>(dst)),
                  "r"(ptx::smem_u32(smem_src)), "r"(bytes)
@@ -419,8 +413,8 @@ evict_kernel(const EvictParams p) {
                             const unsigned stop = (starts | ~movers) & after;
                             const int len = (stop ? __ffs(stop) - 1 : 32) - lane;
                             uint8_t *stage = reinterpret_cast<uint8_t *>(ring_dyn) + st * BR::kStageBytes;
-                            bulk_load(stage + lane * RB, kc + slot_row(src) * kVecPerRow, (uint32_t)len * RB, &full[st]);
-                            bulk_load(stage + (kRows + lane) * RB, vc + slot_row(src) * kVecPerRow, (uint32_t)len * RB,
+                            ptx::bulk_load(stage + lane * RB, kc + slot_row(src) * kVecPerRow, (uint32_t)len * RB, &full[st]);
+                            ptx::bulk_load(stage + (kRows + lane) * RB, vc + slot_row(src) * kVecPerRow, (uint32_t)len * RB,
                                       &full[st]);
                         }
                         if (mv) {

@@ -1,5 +1,5 @@
-// Thin inline-PTX wrappers for sm_100-family features used by the fast decode kernel:
-// mbarriers, tensor-map TMA loads, ldmatrix and bf16 mma.sync.
+// Thin inline-PTX wrappers for sm_100-family features: mbarriers, programmatic dependent launch, cluster
+// barriers, tensor-map TMA and bulk copies, ldmatrix and bf16 mma.sync.
 #pragma once
 
 #include <cuda.h>
@@ -85,6 +85,14 @@ __device__ __forceinline__ void tma_load_2d(void *smem_dst, const CUtensorMap *m
         : "memory");
 }
 
+// 1-D bulk copy of `bytes` into shared memory, completion counted on `bar` (16-byte aligned, size a multiple
+// of 16).
+__device__ __forceinline__ void bulk_load(void *smem_dst, const void *src, uint32_t bytes, uint64_t *bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_u32(smem_dst)),
+                 "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+}
 // Bulk prefetch of [p, p + bytes) into L2 (16-byte aligned, size a multiple of 16).
 __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(reinterpret_cast<uint64_t>(p)), "r"(bytes)

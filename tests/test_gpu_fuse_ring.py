@@ -1,6 +1,6 @@
-"""Stage 1 at the edges of its ring kernels: spans shorter than, equal to and many times a ring stage,
-runs of output rows around a work item's, row widths around a team's columns, short, empty and skipped
-sequences beside long ones. Rows, positions, slot maps and lengths are the oracle's bit for bit. A ring
+"""Stage 1 at the edges of its kernels: spans shorter than, equal to and many times a ring stage,
+runs of output rows around a work item's, embedding widths around the column ranges of a row, short, empty
+and skipped sequences beside long ones. Rows, positions, slot maps and lengths are the oracle's bit for bit. A ring
 whose waits give up leaves every unit that it did not finish empty."""
 import os
 import subprocess

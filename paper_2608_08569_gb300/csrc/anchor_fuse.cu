@@ -429,7 +429,7 @@ fuse_rows_kernel(int32_t B, int32_t L, int32_t Hkv, int32_t C, int32_t stride, i
 // are fuse_rows_kernel's to the last bit.
 // HBM bounds it. The loads of fuse_rows_kernel wait in registers, four rows at most per warp at half an
 // SM's warps; here 192 KB per SM are in flight whatever the spans. voxzip_anchor_fuse as a whole, bf16,
-// D = 128: 4 x 46 024 tokens, 48 layers (25.5 GB) 4.63 -> 3.87 ms, 0.97 of the measured copy rate; 32
+// D = 128: 4 x 46 024 tokens, 48 layers (25.5 GB) 4.63 -> 3.83 ms, 0.98 of the measured copy rate; 32
 // ragged sequences of up to 6 256 tokens 2.96 -> 2.43 ms; one of 8 012 tokens 206 -> 180 us (in fp32 344
 // -> 331); a 30-s clip 45.5 -> 38.5. 16 warps: the sums are issue-bound with fewer (12 warps of four
 // stages 4.46 ms, 8 of six 6.05), and two deep stages for 24 warps run dry (4.24).
